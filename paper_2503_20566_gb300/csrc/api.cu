@@ -25,17 +25,17 @@ enum ScalarKind { S_F32 = 0, S_F64 = 1, S_C64 = 2, S_C128 = 3 };
 
 struct Plan {
   std::vector<int> bondB, bondT, qrB, svdB, qrT, svdT;  // (Ly+1) x (Lx+1) each
-  long long mps_stride = 0, qsite_stride = 0, mat_max = 0, tau_max = 0, tmp_max = 0;
+  long long mps_stride = 0, mat_max = 0, tau_max = 0, tmp_max = 0;
   int env_stride = 0, env3_stride = 0;
   long long ws_stride = 0;
   int ck_every = 0;               // boundary-MPS store: keep every K-th (0: all)
   long long o_Bseg = 0, o_Tseg = 0;
-  long long o_net, o_prop, o_B, o_T, o_Q, o_M1, o_M2, o_M3, o_tau, o_J, o_envR, o_envL, o_envX,
+  long long o_net, o_prop, o_B, o_T, o_Q, o_M1, o_M2, o_M3, o_tau, o_envR, o_envL, o_envX,
       o_envY, o_t1, o_t2, o_t3, o_env3R, o_env3L, o_env3X, o_env3Y, o_G;
   // buffers in dynamic shared memory (elements from the hot base)
   long long o_sigma = 0, o_sel = 0;
   long long so_envR = 0, so_env3R = 0, so_sB = 0, so_sT = 0;
-  long long o_Z = 0, z_size = 0, q_pack = 0, o_X = 0, o_W1 = 0, o_W2 = 0, o_W3 = 0, o_W4 = 0;
+  long long o_Z = 0, o_X = 0, o_W1 = 0, o_W2 = 0, o_W4 = 0;
   long long so_net, so_prop, so_cop, so_envL, so_envX, so_envY, so_env3L, so_env3X, so_env3Y, so_t1,
       so_t2, hot_elems = 0, cfg_bytes = 0;
   size_t dyn_smem = 0;
@@ -351,61 +351,54 @@ void build_plan(gcf_ctx* c) {
     ms = std::max(ms, mps_size(&p.bondT[j * W], j == Ly ? 1 : Dk));
   }
   p.mps_stride = al32(ms);
-  // QR-pass sites, matrices, taus
-  long long qs = 1, mat = 1, tau = 1, fzq = 0, fzj = 0;
+  // Matrices of the absorption (all with columns padded to 4 rows), the
+  // reflectors of a left sweep, the factorisation workspace (see factor.cuh
+  // and truncate_bond): with A the largest absorbed bond of a step, no matrix
+  // has more than A pout rows by A columns (padded), in either orientation.
+  long long mat = 1, tau = 1, qpack = 1;
+  long long fz_vb = 0, fz_w = 0, fz_all = 0;
+  const long long rc = 8 * 16 / (long long)c->sbytes;  // rows of a chunk per lane of 8
+  auto vb = [&](long long m) { return 2 * ((m + rc - 1) / rc * rc) + 4; };
+  auto p4 = [](long long n) { return (n + 3) & ~3LL; };
   bool truncates = false;
-  auto step_sizes = [&](const int* bin, const int* qr, const int* svd, const int* bout, int pin,
-                        int pout) {
-    std::vector<int> ab(Lx + 1);
-    ab[0] = 1;
-    for (int cc = 1; cc < Lx; ++cc) ab[cc] = bin[cc] * Dk;
-    ab[Lx] = 1;
+  auto step_sizes = [&](const int* bin, const int* qr, const int* svd, const int* bout, int pout) {
+    long long A = 1, q = 0;
+    for (int cc = 1; cc < Lx; ++cc) A = std::max(A, (long long)bin[cc] * Dk);
+    mat = std::max(mat, (A * pout + 4) * (A + 8));
+    tau = std::max(tau, A * pout + 4);
     for (int cc = 0; cc < Lx; ++cc) {
-      const long long rows = (long long)qr[cc] * pout, cols = ab[cc + 1];
-      // columns padded to whole 4-row chunks (the FP32 column-major form)
-      fzq = std::max(fzq, ((rows + 3) & ~3LL) * (cols + std::min(rows, cols)));
-      qs = std::max(qs, rows * std::min(rows, cols));
-      mat = std::max(mat, (long long)ab[cc] * pout * ab[cc + 1]);  // Z
-      mat = std::max(mat, rows * cols);                             // X
-      mat = std::max(mat, (long long)std::max(rows, cols) * std::max(rows, cols));
-      tau = std::max(tau, std::max(rows, cols));
-      tau = std::max(tau, (long long)std::max(ab[cc], ab[cc + 1]) * pout);
-    }
-    for (int cc = Lx - 1; cc >= 1; --cc) {
-      const long long yr = qr[cc], yc = (long long)pout * bout[cc + 1];
-      const long long k0 = std::min(yr, yc);
-      fzq = std::max(fzq, ((yc + 3) & ~3LL) * (yr + k0));
-      if (svd[cc]) {
-        truncates = true;
-        // FP32 column-major form: W and J with columns padded to whole 4-row
-        // chunks, the kept columns of J before and after re-orthogonalisation
-        // and their Gram matrix
-        const long long kk = bout[cc], ldj = (k0 + 3) & ~3LL;
-        fzj = std::max(fzj, ((yr + 3) & ~3LL) * k0 + ldj * k0 + 2 * ldj * kk + kk * kk);
+      const long long rows = (long long)qr[cc] * pout, cols = qr[cc + 1];
+      if (rows > cols) {
+        q += (p4(rows) + 1) * cols + 32;
+        fz_vb = std::max(fz_vb, vb(rows));
       }
-      mat = std::max(mat, std::max(yr, yc) * std::max(yr, yc));
-      mat = std::max(mat, k0 * k0);
-      mat = std::max(mat, (long long)qr[cc - 1] * pout * bout[cc]);
-      tau = std::max(tau, std::max(yr, yc));
+      q = (q + 31) & ~31LL;
     }
-    (void)pin;
+    qpack = std::max(qpack, q);
+    for (int cc = Lx - 1; cc >= 1; --cc) {
+      if (!svd[cc]) continue;
+      truncates = true;
+      const long long yr = qr[cc], yc = (long long)pout * bout[cc + 1], k0 = std::min(yr, yc), kk = bout[cc];
+      const long long w = vb(yr) + p4(yc) * ((k0 + 7) & ~7LL);
+      fz_w = std::max(fz_w, w);
+      fz_all = std::max(fz_all, w + p4(yc) * kk + p4(kk * kk));
+    }
   };
   for (int r = 0; r <= Ly - 2; ++r)
-    step_sizes(&p.bondB[r * W], &p.qrB[r * W], &p.svdB[r * W], &p.bondB[(r + 1) * W], r == 0 ? 1 : Dk, Dk);
+    step_sizes(&p.bondB[r * W], &p.qrB[r * W], &p.svdB[r * W], &p.bondB[(r + 1) * W], Dk);
   for (int r = Ly - 1; r >= 1; --r)
-    step_sizes(&p.bondT[(r + 1) * W], &p.qrT[r * W], &p.svdT[r * W], &p.bondT[r * W], r == Ly - 1 ? 1 : Dk, Dk);
-  // shared-memory factorisation workspace: for plans that truncate (the
-  // QR, Q formation and Jacobi sweeps then dominate), the largest of the QR
-  // and Jacobi needs that fits 64 KB; the other runs in global scratch
-  {
-    const long long cap = (64 * 1024) / (long long)c->sbytes;
-    p.fz_elems = 0;
-    if (truncates) {
-      if (fzq <= cap) p.fz_elems = std::max(p.fz_elems, fzq);
-      if (fzj <= cap) p.fz_elems = std::max(p.fz_elems, fzj);
-    }
+    step_sizes(&p.bondT[(r + 1) * W], &p.qrT[r * W], &p.svdT[r * W], &p.bondT[r * W], Dk);
+  // Shared-memory factorisation workspace of plans that truncate: the QR's
+  // reflector buffers, the Jacobi columns and the kept vectors if all fit 64
+  // KB (two chains per SM), else without the kept vectors up to 100 KB (one),
+  // else the reflector buffers alone.
+  p.fz_elems = 0;
+  if (truncates) {
+    const long long sb = (long long)c->sbytes;
+    p.fz_elems = fz_vb;
+    if (fz_all * sb <= 64 * 1024) p.fz_elems = std::max(fz_vb, fz_all);
+    else if (fz_w * sb <= 100 * 1024) p.fz_elems = std::max(fz_vb, fz_w);
   }
-  p.qsite_stride = al32(qs);
   p.mat_max = al32(mat);
   p.tau_max = al32(tau);
   // strip / row environments and intermediates
@@ -474,12 +467,11 @@ void build_plan(gcf_ctx* c) {
     p.o_B = take((Ly + 1) * p.mps_stride);
     p.o_T = take((Ly + 1) * p.mps_stride);
   }
-  p.o_Q = take((long long)Lx * p.qsite_stride);
+  p.o_Q = take(qpack);
   p.o_M1 = take(p.mat_max);
   p.o_M2 = take(p.mat_max);
   p.o_M3 = take(p.mat_max);
   p.o_tau = take(p.tau_max);
-  p.o_J = take(p.mat_max);
   p.o_envR = take((long long)(Lx + 1) * p.env_stride);
   p.o_envL = take(p.env_stride);
   p.o_envX = take(p.env_stride);
@@ -494,7 +486,7 @@ void build_plan(gcf_ctx* c) {
   p.o_G = take(D4);
   p.o_sigma = take(2 * p.tau_max + 32);  // SVD column norms (doubles)
   p.o_sel = take(p.tau_max + 32);         // selected columns (ints)
-  // absorbed sites of one step (warp compression path)
+  // absorbed sites of one step
   long long zmax = 1;
   for (int j = 0; j <= Ly; ++j)
     for (const std::vector<int>* bt : {&p.bondB, &p.bondT}) {
@@ -507,22 +499,10 @@ void build_plan(gcf_ctx* c) {
       }
       zmax = std::max(zmax, z);
     }
-  p.z_size = zmax;
   p.o_Z = take(zmax);
-  // packed QR-pass sites of one step (rows_c x qr[c+1])
-  long long qmax = 1;
-  for (int r = 0; r <= Ly; ++r)
-    for (const std::vector<int>* qt : {&p.qrB, &p.qrT}) {
-      const int* q = &(*qt)[r * W];
-      long long z = 0;
-      for (int cc = 0; cc < Lx; ++cc) z += (long long)q[cc] * Dk * q[cc + 1];
-      qmax = std::max(qmax, z);
-    }
-  p.q_pack = qmax;
   p.o_X = take(p.mat_max);
   p.o_W1 = take(p.mat_max);
   p.o_W2 = take(p.mat_max);
-  p.o_W3 = take(p.mat_max);
   p.o_W4 = take(p.mat_max);
   p.ws_stride = o;
   // hot buffers: shared memory if they fit the budget
@@ -596,12 +576,12 @@ KParams<T> make_params(gcf_ctx* c) {
   k.ws_stride = p.ws_stride;
   k.o_net = p.o_net; k.o_prop = p.o_prop; k.o_B = p.o_B; k.o_T = p.o_T; k.o_Q = p.o_Q;
   k.ck_every = p.ck_every; k.o_Bseg = p.o_Bseg; k.o_Tseg = p.o_Tseg;
-  k.o_M1 = p.o_M1; k.o_M2 = p.o_M2; k.o_M3 = p.o_M3; k.o_tau = p.o_tau; k.o_J = p.o_J;
+  k.o_M1 = p.o_M1; k.o_M2 = p.o_M2; k.o_M3 = p.o_M3; k.o_tau = p.o_tau;
   k.o_envR = p.o_envR; k.o_envL = p.o_envL; k.o_envX = p.o_envX; k.o_envY = p.o_envY;
   k.o_t1 = p.o_t1; k.o_t2 = p.o_t2; k.o_t3 = p.o_t3;
   k.o_env3R = p.o_env3R; k.o_env3L = p.o_env3L; k.o_env3X = p.o_env3X; k.o_env3Y = p.o_env3Y;
   k.o_G = p.o_G;
-  k.mps_stride = p.mps_stride; k.qsite_stride = p.qsite_stride;
+  k.mps_stride = p.mps_stride;
   k.env_stride = p.env_stride; k.env3_stride = p.env3_stride;
   k.max_sweeps_svd = c->svd_sweeps;
   k.hot_in_smem = p.cta_level >= 1;
@@ -609,10 +589,8 @@ KParams<T> make_params(gcf_ctx* c) {
   k.renv_in_smem = p.cta_level >= 3;
   k.so_envR = p.so_envR; k.so_env3R = p.so_env3R; k.so_sB = p.so_sB; k.so_sT = p.so_sT;
   k.o_sigma = p.o_sigma; k.o_sel = p.o_sel;
-  k.dense_max = p.tmp_max;
-  k.o_Z = p.o_Z; k.z_size = p.z_size; k.o_X = p.o_X; k.o_W1 = p.o_W1; k.o_W2 = p.o_W2; k.o_W3 = p.o_W3;
+  k.o_Z = p.o_Z; k.o_X = p.o_X; k.o_W1 = p.o_W1; k.o_W2 = p.o_W2;
   k.o_W4 = p.o_W4;
-  k.q_pack = p.q_pack;
   k.so_net = p.so_net; k.so_prop = p.so_prop; k.so_cop = p.so_cop;
   k.so_envL = p.so_envL; k.so_envX = p.so_envX; k.so_envY = p.so_envY;
   k.so_env3L = p.so_env3L; k.so_env3X = p.so_env3X; k.so_env3Y = p.so_env3Y;
@@ -636,7 +614,6 @@ KParams<T> make_params(gcf_ctx* c) {
   // E_loc); the row environments (amplitude, O, horizontal-hop ratios) run in
   // the 3-pass TF32 form.
   k.row_gemm_mode = k.gemm_mode == GEMM_BF16 ? GEMM_TF32X3 : k.gemm_mode;
-  k.absorb_gemm_mode = GEMM_FFMA;
   k.tc_bf16 = p.tc_bytes > 0 && k.gemm_mode == GEMM_BF16 ? 1 : 0;
   k.tc_bytes = p.tc_bytes;
   k.tc_off = (long long)cta_tc_off(p, p.cta_level, c->sbytes);

@@ -17,6 +17,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "factor.cuh"
 #include "linalg.cuh"
 #include "envsteps.cuh"
 
@@ -52,9 +53,9 @@ struct KParams {
   // scratch
   T* scratch;
   long long ws_stride;     // elements per CTA
-  long long o_net, o_prop, o_B, o_T, o_Q, o_M1, o_M2, o_M3, o_tau, o_J, o_envR, o_envL,
+  long long o_net, o_prop, o_B, o_T, o_Q, o_M1, o_M2, o_M3, o_tau, o_envR, o_envL,
       o_envX, o_envY, o_t1, o_t2, o_t3, o_env3R, o_env3L, o_env3X, o_env3Y, o_G;
-  long long mps_stride, qsite_stride;
+  long long mps_stride;
   // Boundary-MPS store.  ck_every = 0: every B[r] / T[r] of the chain is kept
   // (B slot j at o_B + j mps_stride, T slot r at o_T + r mps_stride).
   // ck_every = K >= 2: only every K-th is kept (B slot j with j % K == 0 at
@@ -69,16 +70,15 @@ struct KParams {
   int max_sweeps_svd;
   // hot buffers: in dynamic shared memory when hot_in_smem, else in scratch
   int hot_in_smem;
-  long long o_sigma, o_sel, dense_max, o_Z, z_size, q_pack, o_X, o_W1, o_W2, o_W3, o_W4;
+  long long o_sigma, o_sel, o_Z, o_X, o_W1, o_W2, o_W4;
   long long so_net, so_prop, so_cop, so_envL, so_envX, so_envY, so_env3L, so_env3X, so_env3Y,
       so_t1, so_t2, smem_cfg_bytes;
   long long group_smem_bytes;  // grouped kernel: shared bytes per chain group
   int group_threads;          // grouped kernel: threads per chain (128)
   int lockstep;               // grouped kernels: keep a CTA's chains at the same row
   int lock_fault;             // test hook: group 0 never counts in, so the others' waits run out
-  int gemm_mode;              // GemmMode of the contraction GEMMs
+  int gemm_mode;              // GemmMode of the environment GEMMs (the absorption keeps the scalar's own precision)
   int row_gemm_mode;          // GemmMode of the row environments (O, amplitude, hops)
-  int absorb_gemm_mode;       // GemmMode of the boundary-MPS absorption (B[r], T[r])
   // BF16 GEMMs of real chains on the fifth-generation tensor cores
   // (tcgen05.cuh): 1 if used, the bytes of a chain's operand staging area and
   // its byte offset from the start of the chain's dynamic shared memory
@@ -218,23 +218,6 @@ __device__ __noinline__ int rescale(const X ex, T* a, int n) {
   return e;
 }
 
-// the same with the scale chosen from the Frobenius norm (|a| -> [0.5, 1))
-template <class T, class X>
-__device__ __noinline__ int frob_rescale(const X ex, T* a, int n) {
-  using R = typename Traits<T>::R;
-  R s2 = R(0);
-#pragma unroll 1
-  for (int i = ex.tid(); i < n; i += ex.size()) s2 += abs2(a[i]);
-  s2 = ex.template sum<R>(s2);
-  if (!(s2 > R(0)) || !isfinite((float)s2)) return 0;
-  const int e = exp2_of((float)sqrt(s2));
-  const R s = pow2r<R>(-e);
-#pragma unroll 1
-  for (int i = ex.tid(); i < n; i += ex.size()) a[i] = scale(a[i], s);
-  ex.sync();
-  return e;
-}
-
 // sum_k A[k] B[k] (no conjugation), broadcast to all threads as (re, im)
 template <class T, class X>
 __device__ __noinline__ void cta_dot(const X ex, const T* A, const T* B, int n, typename Traits<T>::R& r,
@@ -275,7 +258,7 @@ __device__ __noinline__ int dense_absorb(const X ex, const KParams<T>& k, Shared
     const T* M = mps_in + sh.bd_off[c];
     // bufB[(p, i)][b] = sum_a bufA[p][a] M[a][(i b)]
     cta_gemm<T>(ex, rows, pin * bdi[c + 1], bdi[c], bufA, bdi[c], 1, M, pin * bdi[c + 1], 1, bufB,
-                pin * bdi[c + 1], 1, false);
+                pin * bdi[c + 1], 1);
     rows *= pin;
     T* t = bufA; bufA = bufB; bufB = t;
   }
@@ -351,61 +334,99 @@ __device__ inline void select_largest(const X ex, int k0, int kk, const R* sigma
   ex.sync();
 }
 
-// Truncated SVD step of a bond in FP32, in the chain's shared-memory
-// workspace: L (yr x k0, row-major) = W J^T by one-sided Jacobi
-// (jacobi_svd_cm), the kk columns of W with the largest norms kept, one
-// Newton-Schulz step on the kept columns of J only,
-//   Jn = J_s (3 I - J_s^T J_s) / 2,
-// then carry = L Jn (yr x kk, row-major) and site = Jn^T Q'^T (kk x yc,
-// row-major), Q' = Qp (yc x k0, row-major).  The squared column norms of W
-// go to sigma.  Returns false, having done nothing, when the workspace is
-// too small.
-template <class X>
-__device__ __noinline__ bool truncate_f32_smem(const X ex, int yr, int yc, int k0, int kk, const float* L,
-                                               const float* Qp, float* carry, float* site, float* sigma, int* sel,
-                                               int* sflag, int max_sweeps, int* conv) {
-  float* fz = (float*)g_fz[ex.slot()];
-  const int ldw = jac_ld(yr), ldj = jac_ld(k0);
-  if (!fz || (long long)(ldw + ldj) * k0 + 2LL * ldj * kk + (long long)kk * kk > g_fz_elems) return false;
-  float* w = fz;                // W, column-major (ldw)
-  float* jj = w + ldw * k0;     // J, column-major (ldj)
-  float* js = jj + ldj * k0;    // kept columns of J
-  float* jn = js + ldj * kk;    // after the Newton-Schulz step
-  float* gg = jn + ldj * kk;    // kk x kk, row-major
+// The Frobenius norm of a column-major matrix scaled to [0.5, 1) by an exact
+// power of two; the returned integer e means "matrix in = 2^e * matrix out".
+template <class T, class X>
+__device__ __noinline__ int frob_rescale_cm(const X ex, int rows, int cols, T* a, int ld) {
+  using R = typename Traits<T>::R;
+  R s2 = R(0);
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < k0 * ldw; idx += ex.size()) {
-    const int c = idx / ldw, i = idx - (idx / ldw) * ldw;
-    w[idx] = (i < yr) ? L[i * k0 + c] : 0.f;
+  for (int idx = ex.tid(); idx < cols * rows; idx += ex.size()) {
+    const int c = idx / rows, i = idx - (idx / rows) * rows;
+    s2 += abs2(a[c * ld + i]);
+  }
+  s2 = ex.template sum<R>(s2);
+  if (!(s2 > R(0)) || !isfinite((float)s2)) return 0;
+  const int e = exp2_of((float)sqrt(s2));
+  const R s = pow2r<R>(-e);
+#pragma unroll 1
+  for (int idx = ex.tid(); idx < cols * rows; idx += ex.size()) {
+    const int c = idx / rows, i = idx - (idx / rows) * rows;
+    a[c * ld + i] = scale(a[c * ld + i], s);
   }
   ex.sync();
-  jacobi_svd_cm(ex, yr, k0, w, ldw, jj, ldj, sflag, max_sweeps, conv);
+  return e;
+}
+
+// Truncated step of a bond: Y (yr x yc, column-major) ~ carry site, with site
+// the kk x yc (row-major) isometry of Y's kk leading right singular vectors
+// and carry = Y site^H (yr x kk, column-major).  Y = Q R by Householder QR; of
+// it only R is formed, as the columns of W = R^H, whose one-sided Jacobi gives
+// W J = V Sigma: the rotated columns themselves are the right singular vectors
+// of Y, so neither Q nor J is ever needed (R^H, not Y^H, because its columns
+// are closer to orthogonal and converge in fewer sweeps).  The kk columns of
+// largest norm are normalised, and one Newton-Schulz step V (3 I - V^H V) / 2
+// brings them from the sweeps' threshold to orthogonal at rounding.  Columns
+// of norm below eps |Y| are rounding noise, which the sweeps leave alone:
+// their directions are dropped (zero rows of site).
+// Work: W, V and the Gram matrix in the chain's shared-memory workspace as
+// far as they fit it, else in g0, g1, g2 (mat_max each); Vwork, tau for the QR.
+template <class T, class X>
+__device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, const T* Y, int ldy, T* carry, int ldl,
+                                           T* site, T* g0, T* g1, T* g2, T* Vwork, T* tau,
+                                           typename Traits<T>::R* sigma, int* sel, int* sflag, int max_sweeps,
+                                           int* conv) {
+  using R = typename Traits<T>::R;
+  const int k0 = min(yr, yc), kp = (k0 + 7) & ~7, ldw = pad4(yc);
+  const int nvb = qr_vb_elems<T>(yr), nw = ldw * kp, nv = ldw * kk, ng = pad4(kk * kk);
+  T* fz = (T*)g_fz[ex.slot()];
+  long long room = fz ? g_fz_elems : 0;
+  auto place = [&](long long n, T* other) {
+    if (n > room) return other;
+    T* q = fz;
+    fz += n;
+    room -= n;
+    return q;
+  };
+  T* vb = place(nvb, carry);  // the carry is written last
+  T* w = place(nw, g0);
+  T* vs = place(nv, g1);
+  T* gg = place(ng, g2);
 #pragma unroll 1
-  for (int j = ex.tid(); j < k0; j += ex.size()) {
-    const float4* col = reinterpret_cast<const float4*>(w + j * ldw);
-    float s2 = 0.f;
-    for (int q = 0; q < (ldw >> 2); ++q) s2 = dot4(col[q], col[q], s2);
-    sigma[j] = s2;
+  for (int idx = ex.tid(); idx < (kp - k0) * ldw; idx += ex.size()) w[k0 * ldw + idx] = zero<T>();
+  qr_factor<T, true>(ex, yr, yc, Y, ldy, (T*)nullptr, Vwork, ldy, tau, w, ldw, vb);
+  jacobi_columns<T>(ex, yc, kp, w, ldw, sflag, max_sweeps, conv);
+  R f2 = R(0);
+#pragma unroll 1
+  for (int j = ex.warp(); j < k0; j += ex.nwarps()) {
+    R s2 = R(0);
+    for (int i = ex.lane(); i < yc; i += 32) s2 += abs2(w[j * ldw + i]);
+    s2 = warp_sum(s2);
+    if (ex.lane() == 0) {
+      sigma[j] = s2;
+      f2 += s2;
+    }
   }
-  ex.sync();
+  f2 = ex.template sum<R>(f2);
+  const R negl = Traits<T>::eps() * Traits<T>::eps() * f2;
   select_largest(ex, k0, kk, sigma, sel);
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < kk * ldj; idx += ex.size()) {
-    const int n = idx / ldj, i = idx - (idx / ldj) * ldj;
-    js[idx] = jj[sel[n] * ldj + i];
+  for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
+    const int n = idx / yc, i = idx - (idx / yc) * yc;
+    const R s2 = sigma[sel[n]];
+    vs[n * ldw + i] = s2 > negl ? scale(w[sel[n] * ldw + i], R(1) / sqrt(s2)) : zero<T>();
   }
   ex.sync();
-  // gg = J_s^T J_s, then (3 I - gg) / 2
-  tile_gemm_f32(ex, kk, kk, k0, js, ldj, 1, js, 1, ldj, gg, kk, 1);
+  gram_3i<T>(ex, yc, kk, vs, ldw, gg);
+  // V' over W, which is not needed any more
+  cta_gemm_out<T>(ex, yc, kk, kk, vs, 1, ldw, gg, 1, kk, OutMap<T>{w, 1, 1, 0, kk, 0, ldw});
+  cta_gemm_out<T>(ex, yr, kk, yc, Y, 1, ldy, w, 1, ldw, OutMap<T>{carry, 1, 1, 0, kk, 0, ldl});
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < kk * kk; idx += ex.size()) {
-    const int i = idx / kk, j = idx - (idx / kk) * kk;
-    gg[idx] = fmaf(-0.5f, gg[idx], i == j ? 1.5f : 0.f);
+  for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
+    const int n = idx / yc, i = idx - (idx / yc) * yc;
+    site[idx] = conjg(w[n * ldw + i]);
   }
   ex.sync();
-  tile_gemm_f32(ex, k0, kk, kk, js, 1, ldj, gg, kk, 1, jn, 1, ldj);
-  tile_gemm_f32(ex, yr, kk, k0, L, k0, 1, jn, 1, ldj, carry, kk, 1);
-  tile_gemm_f32(ex, kk, yc, k0, jn, ldj, 1, Qp, 1, k0, site, yc, 1);
-  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -417,8 +438,12 @@ __device__ __noinline__ bool truncate_f32_smem(const X ex, int yr, int yc, int k
 //        step's QR left dims and SVD flags.  Returns the binary exponent e of
 //        the scale (output state = 2^e * mout, up to the discarded weight).
 // Algorithm: QR left to right on the absorbed MPS (left-canonical form),
-// then right to left: LQ where no truncation is needed, one-sided Jacobi SVD
-// keeping the chi largest singular values otherwise.
+// then right to left the truncated SVD of every bond above chi.  Where a
+// bond needs no factorisation none is made: a left site with no more rows
+// than columns has the identity as its isometry (its matrix is the carry),
+// and so has a right site whose outer dimensions already fit the bond.  The
+// isometries of the left sweep stay products of reflectors, applied to the
+// carry of the right sweep (kc columns) instead of being formed.
 // ---------------------------------------------------------------------------
 template <class T, class X>
 __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* ws, T* hot_base, Shared& sh, const T* net,
@@ -432,7 +457,6 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   T* M2 = ws + k.o_M2;
   T* M3 = ws + k.o_M3;
   T* tau = ws + k.o_tau;
-  T* Jm = ws + k.o_J;
   T* Qs = ws + k.o_Q;
   int logs = 0;
 #pragma unroll 1
@@ -463,8 +487,10 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
     for (int c = 0; c < Lx; ++c) {
       sh.zoff[c] = zo;
       zo += sh.ab[c] * pout * sh.ab[c + 1];
+      // reflectors and their factors (the isometry of a QR site)
       sh.qoff[c] = qo;
-      qo += qr[c] * pout * qr[c + 1];
+      if (qr[c] * pout > qr[c + 1]) qo += (pad4(qr[c] * pout) + 1) * qr[c + 1] + 32;
+      qo = (qo + 31) & ~31;
     }
     int cl = 0;
     while (cl < Lx - 1 && (any_svd || qr[cl] * pout < sh.ab[cl + 1])) ++cl;
@@ -475,9 +501,8 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   T* Z = ws + k.o_Z;
   T* Xb = ws + k.o_X;
   T* Y = ws + k.o_W1;
-  T* Yh = ws + k.o_W2;
-  T* Qp = ws + k.o_W3;
   T* Lc = ws + k.o_W4;
+  T* Vw = ws + k.o_W2;
   for (int c = 0; c < Lx; ++c) {
     const int a = bdi[c], b = bdi[c + 1];
     const int l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
@@ -499,148 +524,95 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       Zc[idx] = s;
     }
   }
-  // ---- left QR sweep over sites 0..cL-1; R carry in M3 (Rrows x ab[c])
-  if (ex.tid() == 0) M3[0] = one<T>();
+  // ---- left QR sweep over sites 0..cL-1; carry Rc (Rrows x ab[c], column-major)
+  T* Rc = M3;
+  if (ex.tid() == 0) Rc[0] = one<T>();
   ex.sync();
-  int Rrows = 1;
+  int Rrows = 1, ldr = 4, ldxb = 4;
+  T* fz = (T*)g_fz[ex.slot()];
   for (int c = 0; c <= cL; ++c) {
     const int abl = sh.ab[c], abr = sh.ab[c + 1];
-    const int rows = Rrows * pout, cols = abr;
-    // X = R (Rrows x abl) * Z_c (abl x pout*abr) -> (Rrows*pout) x abr
-    T* X = (c == cL) ? Xb : M1;
-    cta_gemm<T>(ex, Rrows, pout * abr, abl, M3, abl, 1, Z + sh.zoff[c], pout * abr, 1, X, pout * abr, 1, false);
+    const int rows = Rrows * pout, cols = abr, ldx = pad4(rows);
+    // Xc = R (Rrows x abl) * Z_c (abl x (pout, abr)) -> (Rrows pout) x abr
+    T* Xc = (c == cL) ? Xb : (Rc == M3 ? M1 : M3);
+    cta_gemm_out<T>(ex, Rrows, pout * abr, abl, Rc, 1, ldr, Z + sh.zoff[c], pout * abr, 1,
+                    OutMap<T>{Xc, 1, pout, 0, abr, 1, ldx});
+    ldxb = ldx;
     if (c == cL) break;
-    const int kq = min(rows, cols);
-    qr_with_q<T>(ex, rows, cols, M1, cols, tau, kq, Qs + sh.qoff[c], kq);
-#pragma unroll 1
-    for (int idx = ex.tid(); idx < kq * cols; idx += ex.size()) {
-      const int i = idx / cols, j = idx - (idx / cols) * cols;
-      M3[idx] = (j >= i) ? M1[i * cols + j] : zero<T>();
+    if (rows <= cols) {
+      Rc = Xc;
+      ldr = ldx;
+      Rrows = rows;
+    } else {
+      T* V = Qs + sh.qoff[c];
+      T* vb = (fz && qr_vb_elems<T>(rows) <= g_fz_elems) ? fz : M2;
+      ldr = pad4(cols);
+      qr_factor<T, false>(ex, rows, cols, Xc, ldx, V, (T*)nullptr, ldx, V + ldx * cols, Rc, ldr, vb);
+      Rrows = cols;
     }
-    ex.sync();
-    logs += frob_rescale(ex, M3, kq * cols);
-    Rrows = kq;
+    logs += frob_rescale_cm(ex, Rrows, cols, Rc, ldr);
   }
-  // ---- right sweep over every site.  The carry Lc (rdim x kc) is the
-  // identity while no bond to the right has been reduced.
+  // ---- right sweep over every site.  The carry Lc (rd x kc, column-major) is
+  // the identity while no bond to the right has been reduced.
+  // Y (cur x (pout, kc), column-major): site c times the carry.
   bool ident = true;
-  int kc = 1, rdim = 1;
+  int kc = 1, ldl = 4;
   for (int c = Lx - 1; c >= 0; --c) {
     const int cur = (c < cL) ? qr[c] : (c == cL ? Rrows : sh.ab[c]);
     const int rd = (c < cL) ? qr[c + 1] : sh.ab[c + 1];
-    const T* S = (c < cL) ? Qs + sh.qoff[c] : (c == cL ? Xb : Z + sh.zoff[c]);
-    const T* Yp;
-    int yc;
-    if (ident) {
-      Yp = S;
-      yc = pout * rd;
+    const int n = ident ? rd : kc, yc = pout * n, ldy = pad4(cur), rows = cur * pout;
+    if (c < cL && rows > rd) {
+      const T* V = Qs + sh.qoff[c];
+      const int ldv = pad4(rows);
+      apply_q<T>(ex, rows, rd, V, ldv, V + ldv * rd, ident ? (const T*)nullptr : Lc, ldl, n, pout, Y, ldy, M1);
+    } else if (c < cL || ident) {
+      // identity isometry (Y = the carry) or identity carry (Y = the site)
+      const T* S = c == cL ? Xb : Z + sh.zoff[c];
+#pragma unroll 1
+      for (int idx = ex.tid(); idx < rows * n; idx += ex.size()) {
+        const int m = idx / rows, q = idx - (idx / rows) * rows;
+        const int i = q / pout, u = q - (q / pout) * pout;
+        T v;
+        if (c < cL) v = ident ? (q == m ? one<T>() : zero<T>()) : Lc[m * ldl + q];
+        else v = c == cL ? S[m * ldxb + q] : S[q * rd + m];
+        Y[(u * n + m) * ldy + i] = v;
+      }
+      ex.sync();
     } else {
-      // Y = S ((cur*pout) x rdim) * Lc (rdim x kc), viewed cur x (pout*kc)
-      cta_gemm<T>(ex, cur * pout, kc, rdim, S, rdim, 1, Lc, kc, 1, Y, kc, 1, false);
-      Yp = Y;
-      yc = pout * kc;
+      const T* S = c == cL ? Xb : Z + sh.zoff[c];
+      cta_gemm_out<T>(ex, rows, n, rd, S, c == cL ? 1 : rd, c == cL ? ldxb : 1, Lc, 1, ldl,
+                      OutMap<T>{Y, pout, 1, n * ldy, n, 0, ldy});
     }
-    const int yr = cur;
     T* site = mout + sh.bd_off2[c];
     if (c >= 1 && (svd[c] || bdo[c] < cur)) {
       const int kk = bdo[c];
-      cta_adjoint<T>(ex, yc, yr, Yp, yc, 1, Yh, yr, 1);
-      const int k0 = min(yr, yc);
-      qr_with_q<T>(ex, yc, yr, Yh, yr, tau, k0, Qp, k0);
-      // L = R'^H (yr x k0)
-#pragma unroll 1
-      for (int idx = ex.tid(); idx < yr * k0; idx += ex.size()) {
-        const int i = idx / k0, j = idx - (idx / k0) * k0;
-        Lc[idx] = (i >= j) ? conjg(Yh[j * yr + i]) : zero<T>();
-      }
-      ex.sync();
       if (!svd[c]) {
-        cta_adjoint<T>(ex, k0, yc, Qp, k0, 1, site, yc, 1);
+        // yc = kk columns already fit the bond: the identity is the isometry
+#pragma unroll 1
+        for (int idx = ex.tid(); idx < kk * yc; idx += ex.size())
+          site[idx] = idx / yc == idx % yc ? one<T>() : zero<T>();
+        T* t = Lc; Lc = Y; Y = t;
+        ldl = ldy;
       } else {
-        // L J = W with orthogonal columns W (one-sided Jacobi).  J is a
-        // product of many rotations, and in FP32 it drifts from orthogonal by
-        // ~1e-5, which enters the kept subspace at every cut; one
-        // Newton-Schulz step J <- J (3 I - J^H J) / 2 restores orthogonality
-        // to rounding, and the kept W = L J is recomputed so that both
-        // factors agree.
         using RR = typename Traits<T>::R;
-        RR* sigma = (RR*)(ws + k.o_sigma);
-        int* sel = (int*)(ws + k.o_sel);
         int conv = 1;
-        bool done = false;
-        if constexpr (std::is_same<T, float>::value)
-          done = truncate_f32_smem(ex, yr, yc, k0, kk, Lc, Qp, Yh, site, sigma, sel, &sh.iflag[0],
-                                   k.max_sweeps_svd, &conv);
-        if (!done) {
-          T* L0 = ws + k.o_M2;
-          T* Gm = ws + k.o_M1;
-          T* Jn = ws + k.o_M3;
-#pragma unroll 1
-          for (int idx = ex.tid(); idx < yr * k0; idx += ex.size()) L0[idx] = Lc[idx];
-          ex.sync();
-          T* fz = (T*)g_fz[ex.slot()];
-          if (fz && (long long)yr * k0 + (long long)k0 * k0 <= g_fz_elems) {
-            // sweeps on shared-memory copies; only J is needed afterwards
-            // (W is recomputed as L J below)
-            T* w = fz;
-            T* jj = fz + yr * k0;
-            cta_copy(ex, yr, k0, Lc, k0, w, k0);
-            cta_jacobi_svd<T>(ex, yr, k0, w, k0, 1, jj, k0, 1, &sh.iflag[0], k.max_sweeps_svd, &conv);
-            cta_copy(ex, k0, k0, jj, k0, Jm, k0);
-          } else {
-            cta_jacobi_svd<T>(ex, yr, k0, Lc, k0, 1, Jm, k0, 1, &sh.iflag[0], k.max_sweeps_svd, &conv);
-          }
-          cta_gemm<T, true, false, false>(ex, k0, k0, k0, Jm, 1, k0, Jm, k0, 1, Gm, k0, 1, false);
-#pragma unroll 1
-          for (int idx = ex.tid(); idx < k0 * k0; idx += ex.size()) {
-            const int i = idx / k0, j = idx - (idx / k0) * k0;
-            Gm[idx] = scale(Gm[idx], RR(-0.5));
-            if (i == j) Gm[idx] += make_scalar<T>(RR(1.5), RR(0));
-          }
-          ex.sync();
-          cta_gemm<T, false, false, false>(ex, k0, k0, k0, Jm, k0, 1, Gm, k0, 1, Jn, k0, 1, false);
-          cta_gemm<T, false, false, false>(ex, yr, k0, k0, L0, k0, 1, Jn, k0, 1, Lc, k0, 1, false);
-          // squared column norms -> sigma, selected columns -> sel (scratch)
-#pragma unroll 1
-          for (int j = ex.tid(); j < k0; j += ex.size()) {
-            RR s2 = RR(0);
-            for (int i = 0; i < yr; ++i) s2 += abs2(Lc[i * k0 + j]);
-            sigma[j] = s2;
-          }
-          ex.sync();
-          select_largest(ex, k0, kk, sigma, sel);
-          // site[n][x] = sum_j conj(J[j][sel n]) Q'^H[j][x]
-#pragma unroll 1
-          for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
-            const int n = idx / yc, x = idx - (idx / yc) * yc;
-            const int jn = sel[n];
-            T s = zero<T>();
-            for (int j = 0; j < k0; ++j) s = fmac(s, conjg(Jn[j * k0 + jn]), conjg(Qp[x * k0 + j]));
-            site[idx] = s;
-          }
-          // carry U S = W[:, sel] (yr x kk)
-#pragma unroll 1
-          for (int idx = ex.tid(); idx < yr * kk; idx += ex.size()) {
-            const int i = idx / kk, n = idx - (idx / kk) * kk;
-            Yh[idx] = Lc[i * k0 + sel[n]];
-          }
-          ex.sync();
-        }
+        ldl = pad4(cur);
+        truncate_bond<T>(ex, cur, yc, kk, Y, ldy, Lc, ldl, site, M1, M2, M3, Vw, tau, (RR*)(ws + k.o_sigma),
+                         (int*)(ws + k.o_sel), &sh.iflag[0], k.max_sweeps_svd, &conv);
         if (!conv && ex.tid() == 0) atomicAdd(&k.status[ST_SVD], 1);
-#pragma unroll 1
-        for (int idx = ex.tid(); idx < yr * kk; idx += ex.size()) Lc[idx] = Yh[idx];
-        ex.sync();
       }
-      logs += frob_rescale(ex, Lc, yr * kk);
+      logs += frob_rescale_cm(ex, cur, kk, Lc, ldl);
       kc = kk;
-      rdim = yr;
       ident = false;
     } else {
       // no reduction at this site's left bond (cur == bdo[c]): keep Y
 #pragma unroll 1
-      for (int idx = ex.tid(); idx < yr * yc; idx += ex.size()) site[idx] = Yp[idx];
+      for (int idx = ex.tid(); idx < cur * yc; idx += ex.size()) {
+        const int i = idx / yc, j = idx - (idx / yc) * yc;
+        site[idx] = Y[j * ldy + i];
+      }
       ex.sync();
-      logs += rescale(ex, site, yr * yc);
+      logs += rescale(ex, site, cur * yc);
       ident = true;
     }
   }

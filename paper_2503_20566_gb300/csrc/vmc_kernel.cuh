@@ -288,8 +288,6 @@ struct Chain {
 
   // ---- boundary MPS --------------------------------------------------------
   __device__ __noinline__ void absorb_B(int r) {  // B[r] = absorb(B[r-1], row r)
-    const bool own_mode = k.absorb_gemm_mode != k.gemm_mode;
-    if (own_mode) set_gemm_mode(k.absorb_gemm_mode);
     const int ls = absorb_compress(ex, k, ws, hot, sv.base, net, Bslot(r), bdB(r), physB(r), r, 0, Bslot(r + 1),
                                       bdB(r + 1), physB(r + 1), qrBt(r), svdBt(r), offBt(r), offBt(r + 1),
                                       denseB(r));
@@ -298,11 +296,8 @@ struct Chain {
       if (k.ck_every && (r + 1) % k.ck_every) sv.segB = (r + 1) / k.ck_every;
     }
     ex.sync();
-    if (own_mode) set_gemm_mode(k.gemm_mode);
   }
   __device__ __noinline__ void absorb_T(int r) {  // T[r] = absorb(T[r+1], row r flipped)
-    const bool own_mode = k.absorb_gemm_mode != k.gemm_mode;
-    if (own_mode) set_gemm_mode(k.absorb_gemm_mode);
     const int ls = absorb_compress(ex, k, ws, hot, sv.base, net, Tslot(r + 1), bdT(r + 1), physT(r + 1), r, 1,
                                       Tslot(r), bdT(r), physT(r), qrTt(r), svdTt(r), offTt(r + 1), offTt(r),
                                       denseT(r));
@@ -311,7 +306,6 @@ struct Chain {
       if (k.ck_every && (k.Ly - r) % k.ck_every) sv.segT = (k.Ly - r) / k.ck_every;
     }
     ex.sync();
-    if (own_mode) set_gemm_mode(k.gemm_mode);
   }
 
   // ---- strip (rows r, r+1) between B[r-1] (slot r) and T[r+2] -------------
