@@ -195,7 +195,8 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
   for (int j = 0; j < min(c0, k); ++j) {
     const T f = conjg(tau[j]);
 #pragma unroll
-    for (int s = 0; s < C; ++s) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp, mask);
+    for (int s = 0; s < C; ++s)
+      if (c0 + s * ngrp < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp, mask);
   }
   if (c0 < k && grp == 0) make_reflector<T, Q>(x[0], c0, nq, li, vb + (c0 & 1) * ldb, tb + (c0 & 1), mask);
 #pragma unroll
@@ -225,7 +226,8 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
             make_reflector<T, Q>(x[s], j + 1, nq, li, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1), mask);
         }
 #pragma unroll
-        for (int s2 = s + 1; s2 < C; ++s2) reflect_col<T, Q>(x[s2], vr, f, q0, mask);
+        for (int s2 = s + 1; s2 < C; ++s2)
+          if (c0 + s2 * ngrp < n) reflect_col<T, Q>(x[s2], vr, f, q0, mask);
       } else {
         if (grp > jj) {
           reflect_col_mem<T, Q>(x[s], v, li, f, q0, ldb, mask);
@@ -292,26 +294,51 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
                                               : zero<T>();
       }
   }
-#pragma unroll 1
-  for (int j = k - 1; j >= 0; --j) {
-    const T* v = V + (long long)j * ldv;
-    const T f = tau[j];
-    const int q0 = j / (8 * E);
-    if constexpr (C > 1) {
-      T vr[Q * E];
+  // v of the next AHEAD steps are under way while one is applied (the reads
+  // come from L2), as far as registers allow; else v is read twice in place
+  constexpr int W = Q * E * (int)sizeof(T) / 4;  // registers of a column
+  constexpr int AHEAD = C * W >= 80 ? 0 : (80 - C * W) / W < 3 ? (80 - C * W) / W : 3;
+  auto fetch = [&](T* r, int j) {
+    const T* v = V + (long long)max(j, 0) * ldv;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int row = E * (li + 8 * q);
-        if (row < mp) load_chunk(vr + q * E, v + row);
-        else {
+    for (int q = 0; q < Q; ++q) {
+      const int row = E * (li + 8 * q);
+      if (row < mp) load_chunk(r + q * E, v + row);
+      else {
 #pragma unroll
-          for (int e = 0; e < E; ++e) vr[q * E + e] = zero<T>();
-        }
+        for (int e = 0; e < E; ++e) r[q * E + e] = zero<T>();
       }
+    }
+  };
+  if constexpr (AHEAD > 0) {
+    T vr[AHEAD][Q * E];
+    T fr[AHEAD];
 #pragma unroll
-      for (int s = 0; s < C; ++s) reflect_col<T, Q>(x[s], vr, f, q0, mask);
-    } else {
-      reflect_col_mem<T, Q>(x[0], v, li, f, q0, mp, mask);
+    for (int a = 0; a < AHEAD; ++a) {
+      fetch(vr[a], k - 1 - a);
+      fr[a] = tau[max(k - 1 - a, 0)];
+    }
+#pragma unroll 1
+    for (int j0 = k - 1; j0 >= 0; j0 -= AHEAD) {
+#pragma unroll
+      for (int a = 0; a < AHEAD; ++a) {
+        const int j = j0 - a;
+        if (j < 0) break;
+        const int q0 = j / (8 * E);
+#pragma unroll
+        for (int s = 0; s < C; ++s)
+          if (s == 0 || c0 + s * ngrp < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0, mask);
+        fetch(vr[a], j - AHEAD);
+        fr[a] = tau[max(j - AHEAD, 0)];
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int j = k - 1; j >= 0; --j) {
+      const T f = tau[j];
+#pragma unroll
+      for (int s = 0; s < C; ++s)
+        if (s == 0 || c0 + s * ngrp < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp, mask);
     }
   }
 #pragma unroll
@@ -438,8 +465,12 @@ __device__ __noinline__ void apply_q(const X ex, int m, int k, const T* V, int l
   const int nq = (m + Chunk<T>::ROWS - 1) / Chunk<T>::ROWS;
   const int ngrp = ex.size() >> 3;
 #define GCF_AQ_CALL(Qv, Cv)                                                                              \
-  for (int c0 = 0; c0 < nc; c0 += Cv * ngrp)                                                             \
-    apply_q_pass<T, Qv, Cv>(ex, m, k, V, ldv, tau, L, ldl, nc, c0, pout, Y, ldy);                        \
+  if (nc <= ngrp) {                                                                                      \
+    apply_q_pass<T, Qv, 1>(ex, m, k, V, ldv, tau, L, ldl, nc, 0, pout, Y, ldy);                          \
+  } else {                                                                                               \
+    for (int c0 = 0; c0 < nc; c0 += Cv * ngrp)                                                           \
+      apply_q_pass<T, Qv, Cv>(ex, m, k, V, ldv, tau, L, ldl, nc, c0, pout, Y, ldy);                      \
+  }                                                                                                      \
   ex.sync();                                                                                             \
   return;
   GCF_QC_CASES(T, GCF_AQ_CALL)
