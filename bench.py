@@ -89,7 +89,7 @@ def load_peaks():
 
 # the files the FP32 sampling kernel is compiled from (its translation unit and
 # every header it includes)
-KERNEL_SOURCES = ("vmc_f32.cu", "launch.h", "common.cuh", "envsteps.cuh", "factor.cuh", "linalg.cuh", "mma.cuh",
+KERNEL_SOURCES = ("vmc_f32.cu", "vmc_cta.cuh", "launch.h", "common.cuh", "envsteps.cuh", "factor.cuh", "linalg.cuh", "mma.cuh",
                   "peps_dev.cuh", "tcgen05.cuh", "vmc_kernel.cuh")
 
 

@@ -11,7 +11,9 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libgcfvmc.so")
-SOURCES = ["api.cu", "init_configs.cu", "sr.cu", "vmc_f32.cu", "vmc_f64.cu", "vmc_c64.cu", "vmc_c128.cu"]
+# the kernels' units first: they take longest
+SOURCES = [f"vmc_{t}{g}.cu" for t in ("c64", "f32", "f64", "c128") for g in ("_group", "")] + ["api.cu", "sr.cu",
+                                                                                              "init_configs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 
@@ -53,7 +55,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
         if verbose and (r.stdout or r.stderr):
             print(r.stdout, r.stderr)
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=max(1, len(jobs))) as ex:
         list(ex.map(run, jobs))
     if force or jobs or _stale(LIB, objs):
         run([exe, *ARCH, "-shared", "-o", LIB, *objs, "-lcudart"])

@@ -783,7 +783,7 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     const size_t gb = (g_tc + area + 15) / 16 * 16;
     bool want4 = fz > 0;
     if (const char* e = std::getenv("GCFVMC_MULTI")) want4 = !std::strcmp(e, "group4");
-    if (want4 && 4 * gb <= 216 * 1024 && occupancy_vmc_multi<T>(512, 4 * gb) >= 1) {
+    if (want4 && 4 * gb <= 216 * 1024 && occupancy_vmc_multi4<T>(4 * gb) >= 1) {
       block = 512;
       group_bytes = (long long)gb;
       smem = 4 * gb;
@@ -797,7 +797,7 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
       }
     }
   }
-  const int per_sm = occupancy_vmc_multi<T>(block, smem);
+  const int per_sm = block == 512 ? occupancy_vmc_multi4<T>(smem) : occupancy_vmc_multi<T>(smem);
   if (per_sm < 1) return fail(c0, GCF_EINVAL, "gcf_sample_multi: the largest context does not fit an SM");
   const int per_cta = block == 512 ? 4 : 1;
   // every resident slot draws from the queue: as many slots as fit, at most
@@ -828,8 +828,12 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
                                c0->stream));
   unsigned long long* d_queue = (unsigned long long*)(d_start + n_ctx + 1);
   CUDA_TRY(c0, cudaMemsetAsync(d_queue, 0, sizeof(unsigned long long), c0->stream));
-  CUDA_TRY(c0, launch_vmc_multi<T>(d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid, block,
-                                   group_bytes, d_queue, smem, c0->stream));
+  if (block == 512)
+    CUDA_TRY(c0, launch_vmc_multi4<T>(d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid, group_bytes,
+                                      d_queue, smem, c0->stream));
+  else
+    CUDA_TRY(c0, launch_vmc_multi<T>(d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid, d_queue, smem,
+                                     c0->stream));
   c0->last_multi_block = block;
   c0->launches += 1;
   std::vector<int> h(4 * n_ctx);
