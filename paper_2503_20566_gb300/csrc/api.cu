@@ -632,13 +632,20 @@ long long balanced_slots(long long n, long long max_slots) {
   return std::max<long long>(1, (n + rounds - 1) / std::max<long long>(1, rounds));
 }
 
+// Threads per CTA of vmc_kernel for n chains: with at most one chain per SM a
+// truncating plan takes 512, since its factorisations and products have work
+// for more than 256 (the results are the same either way; plans that do not
+// truncate lose more in the barriers than they gain).
+int cta_block(const gcf_ctx* c, int n_chains) { return c->plan.fz_elems > 0 && n_chains <= c->sms ? 512 : 256; }
+
 int grid_for(gcf_ctx* c, int n_chains) {
   int per_sm = 1;
+  const int block = cta_block(c, n_chains);
   switch (c->kind) {
-    case S_F32: per_sm = occupancy_vmc<float>(256, c->plan.dyn_smem); break;
-    case S_F64: per_sm = occupancy_vmc<double>(256, c->plan.dyn_smem); break;
-    case S_C64: per_sm = occupancy_vmc<cfloat>(256, c->plan.dyn_smem); break;
-    default: per_sm = occupancy_vmc<cdouble>(256, c->plan.dyn_smem); break;
+    case S_F32: per_sm = occupancy_vmc<float>(block, c->plan.dyn_smem); break;
+    case S_F64: per_sm = occupancy_vmc<double>(block, c->plan.dyn_smem); break;
+    case S_C64: per_sm = occupancy_vmc<cfloat>(block, c->plan.dyn_smem); break;
+    default: per_sm = occupancy_vmc<cdouble>(block, c->plan.dyn_smem); break;
   }
   return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm));
 }
@@ -700,7 +707,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
   if (warp)
     CUDA_TRY(c, launch_vmc_grouped<T>(k, grid, 128 * W, W * c->plan.group_smem, stream));
   else
-    CUDA_TRY(c, launch_vmc<T>(k, grid, 256, c->plan.dyn_smem, stream));
+    CUDA_TRY(c, launch_vmc<T>(k, grid, cta_block(c, n), c->plan.dyn_smem, stream));
   c->launches += 1;
   if (async) return GCF_OK;
   int h_status[4];

@@ -254,6 +254,9 @@ __shared__ int g_gemm_mode[4];
 struct CtaExec {
   __device__ int tid() const { return threadIdx.x; }
   __device__ int size() const { return blockDim.x; }
+  // threads among which the terms of a sum are dealt out: the same for every
+  // block size from 256, so that the results do not depend on it
+  __device__ int sum_size() const { return min((int)blockDim.x, 256); }
   __device__ int lane() const { return threadIdx.x & 31; }
   __device__ int warp() const { return threadIdx.x >> 5; }
   __device__ int nwarps() const { return blockDim.x >> 5; }
@@ -282,6 +285,7 @@ struct GroupExec {
   __device__ int slot() const { return threadIdx.x / G; }
   __device__ int tid() const { return threadIdx.x % G; }
   __device__ int size() const { return G; }
+  __device__ int sum_size() const { return G; }
   __device__ int lane() const { return threadIdx.x & 31; }
   __device__ int warp() const { return (threadIdx.x % G) >> 5; }
   __device__ int nwarps() const { return G >> 5; }
@@ -324,6 +328,12 @@ struct GroupExec {
   }
 };
 
+
+// First term of a thread's share of an n-term sum (stride sum_size).
+template <class X>
+__device__ __forceinline__ int sum_first(const X ex, int n) {
+  return ex.tid() < ex.sum_size() ? ex.tid() : n;
+}
 
 // Streaming store of an output the kernel never reads back (evict-first in
 // L2, so that the chains' scratch stays resident instead).

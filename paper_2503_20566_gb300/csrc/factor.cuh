@@ -589,7 +589,7 @@ __device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int l
   // pairs with one are left as they are
   S f2 = S(0);
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < p * kp; idx += ex.size()) {
+  for (int idx = sum_first(ex, p * kp); idx < p * kp; idx += ex.sum_size()) {
     const int c = idx / p, i = idx - (idx / p) * p;
     f2 += abs2(W[i + (long long)c * ldw]);
   }

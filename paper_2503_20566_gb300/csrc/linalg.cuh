@@ -20,17 +20,22 @@ namespace gcf {
 // Rows of a column-major matrix padded to whole 16-byte chunks of any type.
 __host__ __device__ inline int pad4(int n) { return (n + 3) & ~3; }
 
+// Row offsets of a matrix whose row index may be a pair i = (i / mr, i % mr).
+struct RowMap {
+  int mr, s0, s1;  // row i at (i / mr) s0 + (i % mr) s1
+  __device__ __forceinline__ int operator()(int i) const {
+    const int h = mr == 1 ? i : i / mr;
+    return h * s0 + (i - h * mr) * s1;
+  }
+};
+
 // Address of C(i, j): rows and columns may each be a pair of indices,
 // i = (i / mr, i % mr) and j = (j / nc, j % nc).
 template <class T>
 struct OutMap {
   T* C;
-  int mr, s0, s1;  // row i at (i / mr) s0 + (i % mr) s1
+  RowMap row;
   int nc, s2, s3;  // column j at (j / nc) s2 + (j % nc) s3
-  __device__ __forceinline__ int row(int i) const {
-    const int h = mr == 1 ? i : i / mr;
-    return h * s0 + (i - h * mr) * s1;
-  }
   __device__ __forceinline__ int col(int j) const {
     const int h = j < nc ? 0 : j / nc;
     return h * s2 + (j - h * nc) * s3;
@@ -41,8 +46,8 @@ struct OutMap {
 // memory: each thread accumulates TM x TN tiles of C in registers, summing
 // over k in order.  C must not overlap A or B.
 template <class T, int TM, int TN, class X>
-__device__ __noinline__ void gemm_tiled(const X ex, int M, int N, int K, const T* A, int sAm, int sAk, const T* B,
-                                        int sBk, int sBn, const OutMap<T> out) {
+__device__ __noinline__ void gemm_tiled(const X ex, int M, int N, int K, const T* A, const RowMap ra, int sAk,
+                                        const T* B, int sBk, int sBn, const OutMap<T> out) {
   const int tm = (M + TM - 1) / TM, tn = (N + TN - 1) / TN;
 #pragma unroll 1
   for (int t = ex.tid(); t < tm * tn; t += ex.size()) {
@@ -50,7 +55,7 @@ __device__ __noinline__ void gemm_tiled(const X ex, int M, int N, int K, const T
     const T* ap[TM];
     const T* bp[TN];
 #pragma unroll
-    for (int q = 0; q < TM; ++q) ap[q] = A + min(i0 + q, M - 1) * sAm;  // rows / columns past the edge repeat the last one
+    for (int q = 0; q < TM; ++q) ap[q] = A + ra(min(i0 + q, M - 1));  // rows / columns past the edge repeat the last one
 #pragma unroll
     for (int r = 0; r < TN; ++r) bp[r] = B + min(j0 + r, N - 1) * sBn;
     T acc[TM][TN];
@@ -85,8 +90,8 @@ __device__ __noinline__ void gemm_tiled(const X ex, int M, int N, int K, const T
 // gemm_tiled with the tile that needs the fewest cycles over the executor's
 // threads (per step of k a tile costs its multiply-adds and its loads).
 template <class T, class X>
-__device__ __noinline__ void cta_gemm_out(const X ex, int M, int N, int K, const T* A, int sAm, int sAk, const T* B,
-                                          int sBk, int sBn, const OutMap<T> out) {
+__device__ __noinline__ void cta_gemm_out(const X ex, int M, int N, int K, const T* A, const RowMap ra, int sAk,
+                                          const T* B, int sBk, int sBn, const OutMap<T> out) {
   constexpr int F = Traits<T>::cplx ? 4 : 1;
   const int nt = ex.size();
   auto cost = [&](int tm, int tn) {
@@ -94,9 +99,9 @@ __device__ __noinline__ void cta_gemm_out(const X ex, int M, int N, int K, const
     return ((tiles + nt - 1) / nt) * (F * tm * tn + 2 * (tm + tn));
   };
   const int c44 = cost(4, 4), c42 = cost(4, 2), c22 = cost(2, 2);
-  if (c44 <= c42 && c44 <= c22) gemm_tiled<T, 4, 4>(ex, M, N, K, A, sAm, sAk, B, sBk, sBn, out);
-  else if (c42 <= c22) gemm_tiled<T, 4, 2>(ex, M, N, K, A, sAm, sAk, B, sBk, sBn, out);
-  else gemm_tiled<T, 2, 2>(ex, M, N, K, A, sAm, sAk, B, sBk, sBn, out);
+  if (c44 <= c42 && c44 <= c22) gemm_tiled<T, 4, 4>(ex, M, N, K, A, ra, sAk, B, sBk, sBn, out);
+  else if (c42 <= c22) gemm_tiled<T, 4, 2>(ex, M, N, K, A, ra, sAk, B, sBk, sBn, out);
+  else gemm_tiled<T, 2, 2>(ex, M, N, K, A, ra, sAk, B, sBk, sBn, out);
 }
 
 // C (M x N) = A B in the scalar's own precision (dense absorption).
@@ -275,7 +280,7 @@ __device__ __noinline__ int cta_jacobi(const X ex, int p, int q, T* W, int ldw, 
   // rounding noise of the matrix: pairs with one are left as they are
   R f2 = R(0);
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < p * q; idx += ex.size()) {
+  for (int idx = sum_first(ex, p * q); idx < p * q; idx += ex.sum_size()) {
     const int c = idx / p, i = idx - (idx / p) * p;
     f2 += abs2(W[i + (long long)c * ldw]);
   }

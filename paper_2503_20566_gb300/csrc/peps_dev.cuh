@@ -225,7 +225,7 @@ __device__ __noinline__ void cta_dot(const X ex, const T* A, const T* B, int n, 
   using R = typename Traits<T>::R;
   T s = zero<T>();
 #pragma unroll 1
-  for (int k = ex.tid(); k < n; k += ex.size()) s = fmac(s, A[k], B[k]);
+  for (int k = sum_first(ex, n); k < n; k += ex.sum_size()) s = fmac(s, A[k], B[k]);
   r = re(s);
   i = im(s);
   ex.template sum2<R>(r, i);
@@ -291,7 +291,7 @@ __device__ __noinline__ int dense_absorb(const X ex, const KParams<T>& k, Shared
   const int nv = NU;
   R s2 = R(0);
 #pragma unroll 1
-  for (int i = ex.tid(); i < nv; i += ex.size()) s2 += abs2(bufA[i]);
+  for (int i = sum_first(ex, nv); i < nv; i += ex.sum_size()) s2 += abs2(bufA[i]);
   s2 = ex.template sum<R>(s2);
   const int e = (s2 > R(0) && isfinite((float)s2)) ? exp2_of((float)sqrt(s2)) : 0;
   const R inv = pow2r<R>(-e);
@@ -341,7 +341,7 @@ __device__ __noinline__ int frob_rescale_cm(const X ex, int rows, int cols, T* a
   using R = typename Traits<T>::R;
   R s2 = R(0);
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < cols * rows; idx += ex.size()) {
+  for (int idx = sum_first(ex, cols * rows); idx < cols * rows; idx += ex.sum_size()) {
     const int c = idx / rows, i = idx - (idx / rows) * rows;
     s2 += abs2(a[c * ld + i]);
   }
@@ -356,6 +356,40 @@ __device__ __noinline__ int frob_rescale_cm(const X ex, int rows, int cols, T* a
   }
   ex.sync();
   return e;
+}
+
+// X[(i u)][(b r)] = sum_{l,d} T1[(l d b)][i] W[l][r][d][u] (column-major X, T1
+// with i contiguous): a thread holds the l, d values of one (i, b).
+struct SiteDims {
+  int l, r, pin, pout, sd, su, rows, nb, ldt, ldx;
+};
+template <class T, int DK, class X>
+__device__ __noinline__ void site_product(const X ex, const SiteDims d, const T* W, const T* T1, T* Xc) {
+#pragma unroll 1
+  for (int idx = ex.tid(); idx < d.rows * d.nb; idx += ex.size()) {
+    const int ib = idx / d.rows, i = idx - (idx / d.rows) * d.rows;
+    T t[DK][DK];
+#pragma unroll
+    for (int il = 0; il < DK; ++il)
+#pragma unroll
+      for (int dd = 0; dd < DK; ++dd)
+        t[il][dd] = (il < d.l && dd < d.pin) ? T1[((il * d.pin + dd) * d.nb + ib) * d.ldt + i] : zero<T>();
+#pragma unroll
+    for (int ir = 0; ir < DK; ++ir)
+#pragma unroll
+      for (int iu = 0; iu < DK; ++iu) {
+        if (ir >= d.r || iu >= d.pout) continue;
+        T s = zero<T>();
+#pragma unroll
+        for (int il = 0; il < DK; ++il)
+#pragma unroll
+          for (int dd = 0; dd < DK; ++dd)
+            if (il < d.l && dd < d.pin)
+              s = fmac(s, t[il][dd], W[il * (DK * DK * DK) + ir * (DK * DK) + dd * d.sd + iu * d.su]);
+        Xc[(ib * d.r + ir) * d.ldx + i * d.pout + iu] = s;
+      }
+  }
+  ex.sync();
 }
 
 // Truncated step of a bond: Y (yr x yc, column-major) ~ carry site, with site
@@ -396,18 +430,17 @@ __device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, c
   for (int idx = ex.tid(); idx < (kp - k0) * ldw; idx += ex.size()) w[k0 * ldw + idx] = zero<T>();
   qr_factor<T, true>(ex, yr, yc, Y, ldy, (T*)nullptr, Vwork, ldy, tau, w, ldw, vb);
   jacobi_columns<T>(ex, yc, kp, w, ldw, sflag, max_sweeps, conv);
-  R f2 = R(0);
 #pragma unroll 1
   for (int j = ex.warp(); j < k0; j += ex.nwarps()) {
     R s2 = R(0);
     for (int i = ex.lane(); i < yc; i += 32) s2 += abs2(w[j * ldw + i]);
     s2 = warp_sum(s2);
-    if (ex.lane() == 0) {
-      sigma[j] = s2;
-      f2 += s2;
-    }
+    if (ex.lane() == 0) sigma[j] = s2;
   }
-  f2 = ex.template sum<R>(f2);
+  ex.sync();
+  R f2 = R(0);
+  for (int j = ex.lane(); j < k0; j += 32) f2 += sigma[j];
+  f2 = warp_sum(f2);
   const R negl = Traits<T>::eps() * Traits<T>::eps() * f2;
   select_largest(ex, k0, kk, sigma, sel);
 #pragma unroll 1
@@ -419,8 +452,8 @@ __device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, c
   ex.sync();
   gram_3i<T>(ex, yc, kk, vs, ldw, gg);
   // V' over W, which is not needed any more
-  cta_gemm_out<T>(ex, yc, kk, kk, vs, 1, ldw, gg, 1, kk, OutMap<T>{w, 1, 1, 0, kk, 0, ldw});
-  cta_gemm_out<T>(ex, yr, kk, yc, Y, 1, ldy, w, 1, ldw, OutMap<T>{carry, 1, 1, 0, kk, 0, ldl});
+  cta_gemm_out<T>(ex, yc, kk, kk, vs, {1, 1, 0}, ldw, gg, 1, kk, OutMap<T>{w, {1, 1, 0}, kk, 0, ldw});
+  cta_gemm_out<T>(ex, yr, kk, yc, Y, {1, 1, 0}, ldy, w, 1, ldw, OutMap<T>{carry, {1, 1, 0}, kk, 0, ldl});
 #pragma unroll 1
   for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
     const int n = idx / yc, i = idx - (idx / yc) * yc;
@@ -473,7 +506,7 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
     return dense_absorb<T>(ex, k, sh, net, mps_in, bdi, pin, row, flip, mout, bdo, pout, bufA, bufB);
   }
 
-  // General path.  Z_c (absorbed sites) for all c; then a QR sweep from the
+  // General path.  Z_c (absorbed sites) right of cL; then a QR sweep from the
   // left over the bonds that must shrink (all bonds if the step truncates),
   // then an LQ / truncated-SVD sweep from the right over the bonds that must
   // shrink; sites in between are the absorbed tensors with the carries
@@ -503,7 +536,7 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   T* Y = ws + k.o_W1;
   T* Lc = ws + k.o_W4;
   T* Vw = ws + k.o_W2;
-  for (int c = 0; c < Lx; ++c) {
+  for (int c = cL + 1; c < Lx; ++c) {
     const int a = bdi[c], b = bdi[c + 1];
     const int l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
     const T* M = mps_in + sh.bd_off[c];
@@ -524,19 +557,29 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       Zc[idx] = s;
     }
   }
-  // ---- left QR sweep over sites 0..cL-1; carry Rc (Rrows x ab[c], column-major)
+  // ---- left QR sweep over sites 0..cL-1 (site cL: X only); carry Rc (Rrows x ab[c], column-major)
   T* Rc = M3;
   if (ex.tid() == 0) Rc[0] = one<T>();
   ex.sync();
   int Rrows = 1, ldr = 4, ldxb = 4;
   T* fz = (T*)g_fz[ex.slot()];
   for (int c = 0; c <= cL; ++c) {
-    const int abl = sh.ab[c], abr = sh.ab[c + 1];
-    const int rows = Rrows * pout, cols = abr, ldx = pad4(rows);
-    // Xc = R (Rrows x abl) * Z_c (abl x (pout, abr)) -> (Rrows pout) x abr
+    const int cols = sh.ab[c + 1], rows = Rrows * pout, ldx = pad4(rows);
+    const int nb = bdi[c + 1], l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
+    // X ((Rrows pout) x (b, r)) = sum R[.][(a l)] M[a][d][b] W[l][r][d][u], the
+    // MPS site first: its a bond is the large one
     T* Xc = (c == cL) ? Xb : (Rc == M3 ? M1 : M3);
-    cta_gemm_out<T>(ex, Rrows, pout * abr, abl, Rc, 1, ldr, Z + sh.zoff[c], pout * abr, 1,
-                    OutMap<T>{Xc, 1, pout, 0, abr, 1, ldx});
+    T* T1 = M2;  // [(l d b)][Rrows]
+    const int ldt = pad4(Rrows);
+    cta_gemm_out<T>(ex, l * Rrows, pin * nb, bdi[c], Rc, {Rrows, ldr, 1}, l * ldr, mps_in + sh.bd_off[c], pin * nb, 1,
+                    OutMap<T>{T1, {Rrows, pin * nb * ldt, 1}, pin * nb, 0, ldt});
+    const T* W = net + (long long)(row * Lx + c) * (Dk * Dk * Dk * Dk);
+    const SiteDims sd_{l, r, pin, pout, sd, su, Rrows, nb, ldt, ldx};
+    switch (Dk) {
+      case 1: site_product<T, 1>(ex, sd_, W, T1, Xc); break;
+      case 2: site_product<T, 2>(ex, sd_, W, T1, Xc); break;
+      default: site_product<T, 3>(ex, sd_, W, T1, Xc); break;
+    }
     ldxb = ldx;
     if (c == cL) break;
     if (rows <= cols) {
@@ -580,8 +623,8 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       ex.sync();
     } else {
       const T* S = c == cL ? Xb : Z + sh.zoff[c];
-      cta_gemm_out<T>(ex, rows, n, rd, S, c == cL ? 1 : rd, c == cL ? ldxb : 1, Lc, 1, ldl,
-                      OutMap<T>{Y, pout, 1, n * ldy, n, 0, ldy});
+      cta_gemm_out<T>(ex, rows, n, rd, S, {1, c == cL ? 1 : rd, 0}, c == cL ? ldxb : 1, Lc, 1, ldl,
+                      OutMap<T>{Y, {pout, 1, n * ldy}, n, 0, ldy});
     }
     T* site = mout + sh.bd_off2[c];
     if (c >= 1 && (svd[c] || bdo[c] < cur)) {

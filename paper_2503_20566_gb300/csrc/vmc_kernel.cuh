@@ -975,9 +975,10 @@ __device__ void tc_end(const KParams<T>& k, int n_groups) {
   if (k.tc_bf16) tc_teardown(n_groups);
 }
 
-// One CTA per chain (any size; the general form).
+// One CTA per chain (any size; the general form), of 256 threads (two per SM)
+// or of 512 when there is at most one chain per SM.
 template <class T>
-__global__ void __launch_bounds__(256, 2) vmc_kernel(const __grid_constant__ KParams<T> k) {
+__global__ void __launch_bounds__(512, 1) vmc_kernel(const __grid_constant__ KParams<T> k) {
   extern __shared__ __align__(16) int8_t dyn_smem[];
   int8_t* dyn_cfg = dyn_smem;
   T* hot = (T*)(dyn_smem + k.smem_cfg_bytes);
