@@ -12,7 +12,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libgcfvmc.so")
 # the kernels' units first: they take longest
-SOURCES = [f"vmc_{t}{g}.cu" for t in ("c64", "f32", "f64", "c128") for g in ("_group", "")] + ["api.cu", "sr.cu",
+SOURCES = [f"vmc_{t}{g}.cu" for t in ("c64", "f32", "f32_tc", "f64", "c128") for g in ("_group", "")] + ["api.cu", "sr.cu",
                                                                                               "init_configs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

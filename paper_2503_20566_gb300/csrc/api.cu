@@ -10,6 +10,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/gcfvmc.h"
@@ -229,7 +230,7 @@ void plan_group(gcf_ctx* c) {
   // two groups per CTA: the largest level that leaves room for a second CTA
   int lv2 = 0;
   for (int lv = 1; lv <= 3; ++lv)
-    if (fits(2, lv, 110 * 1024)) lv2 = lv;
+    if (fits(2, lv, 98 * 1024)) lv2 = lv;
   // Default form: four chain groups per CTA of 512 threads (one CTA per SM)
   // in lockstep, with the hot buffers in shared memory (level 1; the larger
   // levels measured slower for four groups); else two groups per CTA; else
@@ -540,8 +541,9 @@ void build_plan(gcf_ctx* c) {
     const int Nmax = Dk * Dk * chib, Kmax = Dk * chib;
     if (Nmax <= 128) p.tc_bytes = (tc_stage_bytes(Nmax, Kmax) + 15) / 16 * 16;
   }
-  // one chain per CTA: the largest level that keeps two CTAs on an SM
-  const size_t budget = 100 * 1024;
+  // one chain per CTA: the largest level that keeps two CTAs on an SM (113 KB
+  // each, 16 KB of it static)
+  const size_t budget = 96 * 1024;
   p.cta_level = 0;
   for (int lv = 1; lv <= 3; ++lv)
     if (cta_smem_bytes(p, lv, c->sbytes) <= budget) p.cta_level = lv;
@@ -632,6 +634,16 @@ long long balanced_slots(long long n, long long max_slots) {
   return std::max<long long>(1, (n + rounds - 1) / std::max<long long>(1, rounds));
 }
 
+// The launchers and occupancy queries of launch.h in the variant that the
+// context's form needs: with tcgen05 for a BF16 context that uses it.
+bool uses_tc(const gcf_ctx* c) { return c->plan.tc_bytes > 0; }
+#define GCF_TC_CALL(T, tc, fn, ...)                                       \
+  [&] {                                                                   \
+    if constexpr (std::is_same<T, float>::value)                          \
+      if (tc) return fn<T, std::is_same<T, float>::value>(__VA_ARGS__);   \
+    return fn<T, false>(__VA_ARGS__);                                     \
+  }()
+
 // Threads per CTA of vmc_kernel for n chains: with at most one chain per SM a
 // truncating plan takes 512, since its factorisations and products have work
 // for more than 256 (the results are the same either way; plans that do not
@@ -642,10 +654,10 @@ int grid_for(gcf_ctx* c, int n_chains) {
   int per_sm = 1;
   const int block = cta_block(c, n_chains);
   switch (c->kind) {
-    case S_F32: per_sm = occupancy_vmc<float>(block, c->plan.dyn_smem); break;
-    case S_F64: per_sm = occupancy_vmc<double>(block, c->plan.dyn_smem); break;
-    case S_C64: per_sm = occupancy_vmc<cfloat>(block, c->plan.dyn_smem); break;
-    default: per_sm = occupancy_vmc<cdouble>(block, c->plan.dyn_smem); break;
+    case S_F32: per_sm = GCF_TC_CALL(float, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
+    case S_F64: per_sm = GCF_TC_CALL(double, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
+    case S_C64: per_sm = GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
+    default: per_sm = GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
   }
   return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm));
 }
@@ -679,7 +691,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
   const int W = n_groups(c);  // chains per CTA
   int grid = 1;
   if (warp) {
-    const int per_sm = occupancy_vmc_grouped<T>(128 * W, W * c->plan.group_smem);
+    const int per_sm = GCF_TC_CALL(T, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem);
     if (per_sm < 1) return fail(c, GCF_EINVAL, "grouped launch does not fit an SM");
     const long long slots = balanced_slots(n, (long long)c->sms * per_sm * W);
     grid = (int)std::max<long long>(1, (slots + W - 1) / W);
@@ -705,9 +717,9 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
   }
   CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), stream));
   if (warp)
-    CUDA_TRY(c, launch_vmc_grouped<T>(k, grid, 128 * W, W * c->plan.group_smem, stream));
+    CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc_grouped, k, grid, 128 * W, W * c->plan.group_smem, stream));
   else
-    CUDA_TRY(c, launch_vmc<T>(k, grid, cta_block(c, n), c->plan.dyn_smem, stream));
+    CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc, k, grid, cta_block(c, n), c->plan.dyn_smem, stream));
   c->launches += 1;
   if (async) return GCF_OK;
   int h_status[4];
@@ -790,7 +802,7 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     const size_t gb = (g_tc + area + 15) / 16 * 16;
     bool want4 = fz > 0;
     if (const char* e = std::getenv("GCFVMC_MULTI")) want4 = !std::strcmp(e, "group4");
-    if (want4 && 4 * gb <= 216 * 1024 && occupancy_vmc_multi4<T>(4 * gb) >= 1) {
+    if (want4 && 4 * gb <= 216 * 1024 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi4, 4 * gb) >= 1) {
       block = 512;
       group_bytes = (long long)gb;
       smem = 4 * gb;
@@ -804,7 +816,8 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
       }
     }
   }
-  const int per_sm = block == 512 ? occupancy_vmc_multi4<T>(smem) : occupancy_vmc_multi<T>(smem);
+  const int per_sm = block == 512 ? GCF_TC_CALL(T, tc_all, occupancy_vmc_multi4, smem)
+                                  : GCF_TC_CALL(T, tc_all, occupancy_vmc_multi, smem);
   if (per_sm < 1) return fail(c0, GCF_EINVAL, "gcf_sample_multi: the largest context does not fit an SM");
   const int per_cta = block == 512 ? 4 : 1;
   // every resident slot draws from the queue: as many slots as fit, at most
@@ -836,11 +849,11 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
   unsigned long long* d_queue = (unsigned long long*)(d_start + n_ctx + 1);
   CUDA_TRY(c0, cudaMemsetAsync(d_queue, 0, sizeof(unsigned long long), c0->stream));
   if (block == 512)
-    CUDA_TRY(c0, launch_vmc_multi4<T>(d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid, group_bytes,
-                                      d_queue, smem, c0->stream));
+    CUDA_TRY(c0, GCF_TC_CALL(T, tc_all, launch_vmc_multi4, d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid,
+                             group_bytes, d_queue, smem, c0->stream));
   else
-    CUDA_TRY(c0, launch_vmc_multi<T>(d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid, d_queue, smem,
-                                     c0->stream));
+    CUDA_TRY(c0, GCF_TC_CALL(T, tc_all, launch_vmc_multi, d_ks, n_ctx, d_start, total, (T*)c0->multi_arena, ws, (int)grid,
+                             d_queue, smem, c0->stream));
   c0->last_multi_block = block;
   c0->launches += 1;
   std::vector<int> h(4 * n_ctx);
@@ -1375,10 +1388,10 @@ gcf_status gcf_sample_batch_async(gcf_ctx* c, int n_chains, int n_sweeps, uint64
     if (grp) {
       int per_sm = 0;
       switch (c->kind) {
-        case S_F32: per_sm = occupancy_vmc_grouped<float>(128 * W, W * c->plan.group_smem); break;
-        case S_F64: per_sm = occupancy_vmc_grouped<double>(128 * W, W * c->plan.group_smem); break;
-        case S_C64: per_sm = occupancy_vmc_grouped<cfloat>(128 * W, W * c->plan.group_smem); break;
-        default: per_sm = occupancy_vmc_grouped<cdouble>(128 * W, W * c->plan.group_smem); break;
+        case S_F32: per_sm = GCF_TC_CALL(float, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
+        case S_F64: per_sm = GCF_TC_CALL(double, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
+        case S_C64: per_sm = GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
+        default: per_sm = GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
       }
       const long long sl = balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm) * W);
       slots = (sl + W - 1) / W * W;
@@ -1569,7 +1582,7 @@ gcf_status amplitude_noalloc_impl(gcf_ctx* c, int n, const int8_t* configs, doub
   // previous call's values otherwise); the kernel writes every scratch word
   // it reads before reading it
   CUDA_TRY(c, cudaMemsetAsync(status, 0, 4 * sizeof(int), c->stream));
-  CUDA_TRY(c, launch_vmc<T>(k, grid, 256, c->plan.dyn_smem, c->stream));
+  CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc, k, grid, 256, c->plan.dyn_smem, c->stream));
   c->launches += 1;
   return GCF_OK;
 }

@@ -251,7 +251,16 @@ __shared__ double g_exec_red[4][64];
 // own slot between passes.
 __shared__ int g_gemm_mode[4];
 
-struct CtaExec {
+//
+// TC: the executor of a kernel whose environment GEMMs may run on tcgen05 (the
+// BF16 form).  A kernel that holds tcgen05 instructions is given one block
+// per SM whatever its resources (the occupancy query's answer, and the
+// launches' behaviour: 118 -> 64 ms is what the second block is worth to 304
+// log-derivatives at 16x16, chi = 24), so the other forms' kernels are
+// compiled without them.
+template <bool TC = false>
+struct CtaExecT {
+  static constexpr bool tc = TC;
   __device__ int tid() const { return threadIdx.x; }
   __device__ int size() const { return blockDim.x; }
   // threads among which the terms of a sum are dealt out: the same for every
@@ -278,8 +287,11 @@ struct CtaExec {
   }
 };
 
-template <int G>
+using CtaExec = CtaExecT<false>;
+
+template <int G, bool TC = false>
 struct GroupExec {
+  static constexpr bool tc = TC;
   static_assert(G % 32 == 0 && G >= 64 && G <= 128, "group of 64 or 128 threads");
   __device__ int group() const { return threadIdx.x / G; }
   __device__ int slot() const { return threadIdx.x / G; }

@@ -94,7 +94,7 @@ __device__ __noinline__ int cta_gemm_scaled(const X ex, int M, int N, int K, con
   const int MN = M * N;
   const int nt = ex.size();
   bool done = false;
-  if constexpr (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, float>::value && X::tc) {
     // BF16 form of a real chain: the fifth-generation tensor cores when the
     // launch set them up and the operands fit the chain's staging area
     const int slot = ex.slot();

@@ -51,24 +51,25 @@ __device__ __forceinline__ void store_chunk(T* p, const T* x) {
   *reinterpret_cast<float4*>(p) = u.v;
 }
 
-// Sum over the 8 lanes of a column (all lanes of the group call; `mask` the
-// group's lanes).
+// Sum over the 8 lanes of a column.  Every lane of the warp calls it: a warp's
+// four columns take all branches together (a shuffle under a mask of 8 lanes
+// would run the four one after the other).
 template <class R>
-__device__ __forceinline__ R sum8(R v, unsigned mask) {
-  v += __shfl_xor_sync(mask, v, 4);
-  v += __shfl_xor_sync(mask, v, 2);
-  v += __shfl_xor_sync(mask, v, 1);
+__device__ __forceinline__ R sum8(R v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
   return v;
 }
-__device__ __forceinline__ float sum8s(float v, unsigned m) { return sum8(v, m); }
-__device__ __forceinline__ double sum8s(double v, unsigned m) { return sum8(v, m); }
-__device__ __forceinline__ cfloat sum8s(cfloat v, unsigned m) { return {sum8(v.x, m), sum8(v.y, m)}; }
-__device__ __forceinline__ cdouble sum8s(cdouble v, unsigned m) { return {sum8(v.x, m), sum8(v.y, m)}; }
+__device__ __forceinline__ float sum8s(float v) { return sum8(v); }
+__device__ __forceinline__ double sum8s(double v) { return sum8(v); }
+__device__ __forceinline__ cfloat sum8s(cfloat v) { return {sum8(v.x), sum8(v.y)}; }
+__device__ __forceinline__ cdouble sum8s(cdouble v) { return {sum8(v.x), sum8(v.y)}; }
 
 // x <- x - f v (v^H x) on the 8 lanes of a column, v in registers; the chunks
 // q < q0 of v are zero.
 template <class T, int Q>
-__device__ __forceinline__ void reflect_col(T* x, const T* vr, T f, int q0, unsigned mask) {
+__device__ __forceinline__ void reflect_col(T* x, const T* vr, T f, int q0) {
   constexpr int E = Chunk<T>::E;
   T w0 = zero<T>(), w1 = zero<T>();
 #pragma unroll
@@ -80,7 +81,7 @@ __device__ __forceinline__ void reflect_col(T* x, const T* vr, T f, int q0, unsi
         else w0 = fmac(w0, conjg(vr[q * E + e]), x[q * E + e]);
       }
     }
-  const T g = -(f * sum8s(w0 + w1, mask));
+  const T g = -(f * sum8s(w0 + w1));
 #pragma unroll
   for (int q = 0; q < Q; ++q)
     if (Q < 3 || q >= q0) {
@@ -91,7 +92,7 @@ __device__ __forceinline__ void reflect_col(T* x, const T* vr, T f, int q0, unsi
 // The same with v read from memory (its first `lim` rows, whole chunks) twice,
 // for columns too long to hold v beside x.
 template <class T, int Q>
-__device__ __forceinline__ void reflect_col_mem(T* x, const T* v, int li, T f, int q0, int lim, unsigned mask) {
+__device__ __forceinline__ void reflect_col_mem(T* x, const T* v, int li, T f, int q0, int lim) {
   constexpr int E = Chunk<T>::E;
   T w0 = zero<T>(), w1 = zero<T>();
 #pragma unroll
@@ -105,7 +106,7 @@ __device__ __forceinline__ void reflect_col_mem(T* x, const T* v, int li, T f, i
         else w0 = fmac(w0, conjg(c[e]), x[q * E + e]);
       }
     }
-  const T g = -(f * sum8s(w0 + w1, mask));
+  const T g = -(f * sum8s(w0 + w1));
   asm volatile("" ::: "memory");  // read v again rather than hold it
 #pragma unroll
   for (int q = 0; q < Q; ++q)
@@ -119,9 +120,10 @@ __device__ __forceinline__ void reflect_col_mem(T* x, const T* v, int li, T f, i
 
 // Reflector of column j held in x (rows E (li + 8 q) + e of the lane):
 // publishes v (1 at row j, zero above) to vb and tau to *tb, and leaves
-// beta and v below it in x.  The 8 lanes of the column call it.
+// beta and v below it in x.  All lanes of the column's warp call it; only
+// the column's own (`own`) publish and change x.
 template <class T, int Q>
-__device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, T* vb, T* tb, unsigned mask) {
+__device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, bool own, T* vb, T* tb) {
   using R = typename Traits<T>::R;
   constexpr int E = Chunk<T>::E;
   R p0 = R(0), p1 = R(0);
@@ -136,24 +138,27 @@ __device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, T* v
       else p0 += a;
       if (row == j) al = x[q * E + e];
     }
-  const R xn2 = sum8(p0 + p1, mask);
-  al = sum8s(al, mask);
+  const R xn2 = sum8(p0 + p1);
+  al = sum8s(al);
   T t, sc, beta;
-  householder(al, xn2, t, sc, beta);
+  householder_fast(al, xn2, t, sc, beta);
+  if (own) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    if (q >= nq) continue;
-    T c[E];
+    for (int q = 0; q < Q; ++q) {
+      if (q >= nq) continue;
+      T c[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int row = E * (li + 8 * q) + e;
-      const T s = x[q * E + e] * sc;
-      c[e] = row < j ? zero<T>() : row == j ? one<T>() : s;
-      x[q * E + e] = row < j ? x[q * E + e] : row == j ? beta : s;
+      for (int e = 0; e < E; ++e) {
+        const int row = E * (li + 8 * q) + e;
+        const T s = x[q * E + e] * sc;
+        c[e] = row < j ? zero<T>() : row == j ? one<T>() : s;
+        x[q * E + e] = row < j ? x[q * E + e] : row == j ? beta : s;
+      }
+      store_chunk(vb + E * (li + 8 * q), c);
     }
-    store_chunk(vb + E * (li + 8 * q), c);
+    if (li == 0) *tb = t;
   }
-  if (li == 0) *tb = t;
+  __syncwarp();
 }
 
 // One register pass of the Householder QR of A (m x n, column-major): columns
@@ -171,7 +176,6 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
                                      T* Rt, int ldr, T* vb) {
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
-  const unsigned mask = 0xffu << (ex.lane() & 24);
   const int k = min(m, n), mp = (m + E - 1) / E * E, ldb = (m + 8 * E - 1) / (8 * E) * (8 * E), nq = ldb / (8 * E);
   T* tb = vb + 2 * ldb;
   T x[C][Q * E];
@@ -196,9 +200,10 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
     const T f = conjg(tau[j]);
 #pragma unroll
     for (int s = 0; s < C; ++s)
-      if (c0 + s * ngrp < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp, mask);
+      if (c0 + s * ngrp < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
   }
-  if (c0 < k && grp == 0) make_reflector<T, Q>(x[0], c0, nq, li, vb + (c0 & 1) * ldb, tb + (c0 & 1), mask);
+  if (c0 < k && ex.warp() == 0)
+    make_reflector<T, Q>(x[0], c0, nq, li, grp == 0, vb + (c0 & 1) * ldb, tb + (c0 & 1));
 #pragma unroll
   for (int s = 0; s < C; ++s) {
 #pragma unroll 1
@@ -220,24 +225,20 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
             for (int e = 0; e < E; ++e) vr[q * E + e] = zero<T>();
           }
         }
-        if (grp > jj) {
-          reflect_col<T, Q>(x[s], vr, f, q0, mask);
-          if (grp == jj + 1 && j + 1 < k)
-            make_reflector<T, Q>(x[s], j + 1, nq, li, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1), mask);
-        }
+        reflect_col<T, Q>(x[s], vr, grp > jj ? f : zero<T>(), q0);
+        if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
+          make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
 #pragma unroll
         for (int s2 = s + 1; s2 < C; ++s2)
-          if (c0 + s2 * ngrp < n) reflect_col<T, Q>(x[s2], vr, f, q0, mask);
+          if (c0 + s2 * ngrp < n) reflect_col<T, Q>(x[s2], vr, f, q0);
       } else {
-        if (grp > jj) {
-          reflect_col_mem<T, Q>(x[s], v, li, f, q0, ldb, mask);
-          if (grp == jj + 1 && j + 1 < k)
-            make_reflector<T, Q>(x[s], j + 1, nq, li, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1), mask);
-        }
+        reflect_col_mem<T, Q>(x[s], v, li, grp > jj ? f : zero<T>(), q0, ldb);
+        if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
+          make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
       }
-      if (s + 1 < C && jj == ngrp - 1 && grp == 0 && j + 1 < k)
-        make_reflector<T, Q>(x[s + 1 < C ? s + 1 : s], j + 1, nq, li, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1),
-                             mask);
+      if (s + 1 < C && jj == ngrp - 1 && ex.warp() == 0 && j + 1 < k)
+        make_reflector<T, Q>(x[s + 1 < C ? s + 1 : s], j + 1, nq, li, grp == 0, vb + ((j + 1) & 1) * ldb,
+                             tb + ((j + 1) & 1));
     }
   }
 #pragma unroll
@@ -279,7 +280,6 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
                                           int ldl, int nc, int c0, int pout, T* Y, int ldy) {
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
-  const unsigned mask = 0xffu << (ex.lane() & 24);
   const int mp = (m + E - 1) / E * E;
   T x[C][Q * E];
 #pragma unroll
@@ -327,7 +327,7 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
         const int q0 = j / (8 * E);
 #pragma unroll
         for (int s = 0; s < C; ++s)
-          if (s == 0 || c0 + s * ngrp < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0, mask);
+          if (s == 0 || c0 + s * ngrp < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0);
         fetch(vr[a], j - AHEAD);
         fr[a] = tau[max(j - AHEAD, 0)];
       }
@@ -338,7 +338,7 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
       const T f = tau[j];
 #pragma unroll
       for (int s = 0; s < C; ++s)
-        if (s == 0 || c0 + s * ngrp < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp, mask);
+        if (s == 0 || c0 + s * ngrp < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
     }
   }
 #pragma unroll
@@ -524,16 +524,25 @@ __device__ __forceinline__ bool pair_rotation(typename Traits<T>::R& al, typenam
   c = R(1);
   se = zero<T>();
   const R gr = re(g), gi = im(g);
-  const R ga = Traits<T>::cplx ? sqrt(gr * gr + gi * gi) : fabs(gr);
+  R ga, iga;
+  if constexpr (Traits<T>::cplx) {
+    const R g2 = gr * gr + gi * gi;
+    iga = jrsqrt1(g2);
+    ga = g2 * iga;
+    if (!(g2 > R(0))) return false;
+  } else {
+    ga = fabs(gr);
+    iga = jrcpa(ga);
+    if (ga == R(0)) return false;
+  }
   // sqrt(al) sqrt(be), not sqrt(al be): the product of two small squared norms can underflow
-  if (ga == R(0) || !(al > negl) || !(be > negl) || !(ga > tol * (sqrt(al) * sqrt(be)))) return false;
-  const R iga = jrcp(ga);
+  if (!(al > negl) || !(be > negl) || !(ga > tol * (jsqrta(al) * jsqrta(be)))) return false;
   const R zeta = (be - al) * (R(0.5) * iga);
   const R az = fabs(zeta);
   // for |zeta| beyond 1e15, zeta^2 would overflow in FP32, and t = 1 / (2 zeta) to rounding
-  const R t = (zeta >= R(0) ? R(1) : R(-1)) * jrcp(az > R(1e15) ? R(2) * az : az + sqrt(R(1) + zeta * zeta));
+  const R t = (zeta >= R(0) ? R(1) : R(-1)) * jrcpa(az > R(1e15) ? R(2) * az : az + jsqrta(R(1) + zeta * zeta));
   if (t == R(0)) return false;
-  c = jrsqrt(R(1) + t * t);
+  c = jrsqrt1(R(1) + t * t);  // c^2 + s^2 = 1 to rounding whatever the error of t
   const R s = c * t;
   if constexpr (Traits<T>::cplx) se = make_scalar<T>(s * (gr * iga), s * (gi * iga));
   else se = gr >= R(0) ? s : -s;

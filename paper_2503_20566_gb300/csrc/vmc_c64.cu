@@ -1,4 +1,4 @@
 // One-chain-per-CTA kernels for scalar type cfloat.
 #include "vmc_cta.cuh"
 
-GCF_INSTANTIATE_CTA(cfloat)
+GCF_INSTANTIATE_CTA(cfloat, false)

@@ -1,4 +1,4 @@
 // Kernels with several chains per CTA for scalar type double.
 #include "vmc_group.cuh"
 
-GCF_INSTANTIATE_GROUP(double)
+GCF_INSTANTIATE_GROUP(double, false)

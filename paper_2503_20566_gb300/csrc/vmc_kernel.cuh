@@ -950,7 +950,7 @@ __device__ void run_chain(const X ex, const KParams<T>& k, T* ws, SharedV& sv, i
 // completion barrier per chain group, and each group's operand staging area
 // at byte `tc_off` of the group's dynamic shared memory (group g's region
 // starts at g * group_bytes).  Every thread of the CTA calls it.
-template <class T>
+template <class T, bool TC>
 __device__ void tc_begin(const KParams<T>& k, int n_groups, int8_t* dyn_base, long long group_bytes) {
   if (threadIdx.x < 4)
     g_tc_stage[threadIdx.x] = (k.tc_bf16 && threadIdx.x < n_groups)
@@ -965,50 +965,50 @@ __device__ void tc_begin(const KParams<T>& k, int n_groups, int8_t* dyn_base, lo
     g_tc_status = k.status + ST_TC_TIMEOUT;
     g_fz_elems = k.fz_elems;
   }
-  if (k.tc_bf16) tc_setup(n_groups);
+  if constexpr (TC) tc_setup(n_groups);
   bulk_setup(n_groups);
 }
-template <class T>
+template <class T, bool TC>
 __device__ void tc_end(const KParams<T>& k, int n_groups) {
   __syncthreads();
   bulk_teardown(n_groups);
-  if (k.tc_bf16) tc_teardown(n_groups);
+  if constexpr (TC) tc_teardown(n_groups);
 }
 
 // One CTA per chain (any size; the general form), of 256 threads (two per SM)
 // or of 512 when there is at most one chain per SM.
-template <class T>
+template <class T, bool TC>
 __global__ void __launch_bounds__(512, 1) vmc_kernel(const __grid_constant__ KParams<T> k) {
   extern __shared__ __align__(16) int8_t dyn_smem[];
   int8_t* dyn_cfg = dyn_smem;
   T* hot = (T*)(dyn_smem + k.smem_cfg_bytes);
   __shared__ SharedV sv;
-  CtaExec ex;
+  CtaExecT<TC> ex;
   if (threadIdx.x < 4) g_gemm_mode[threadIdx.x] = k.gemm_mode;
   const int* tab = stage_tables(k);
-  tc_begin(k, 1, dyn_smem, 0);
+  tc_begin<T, TC>(k, 1, dyn_smem, 0);
   T* ws = k.scratch + (long long)blockIdx.x * k.ws_stride;
   init_trivial_slots(ex, k, ws);
   for (int chain = blockIdx.x; chain < k.n_chains; chain += gridDim.x)
     run_chain(ex, k, ws, sv, dyn_cfg, hot, tab, chain);
-  tc_end(k, 1);
+  tc_end<T, TC>(k, 1);
 }
 
 // Several chains per CTA, one per group of G = 128 threads (GroupExec, a
 // hardware barrier per group).  Groups never wait on one another.  Dynamic
 // shared memory per group: [SharedV][configuration][hot buffers].
-template <class T, class X, int G>
+template <class T, bool TC, int G>
 __device__ void grouped_body(const KParams<T>& k) {
   extern __shared__ __align__(16) int8_t dyn_smem[];
   if (threadIdx.x < 4) g_gemm_mode[threadIdx.x] = k.gemm_mode;
   const int* tab = stage_tables(k);
   const int g = threadIdx.x / G, NG = blockDim.x / G;
-  tc_begin(k, NG, dyn_smem, k.group_smem_bytes);
+  tc_begin<T, TC>(k, NG, dyn_smem, k.group_smem_bytes);
   int8_t* base = dyn_smem + g * k.group_smem_bytes;
   SharedV& sv = *reinterpret_cast<SharedV*>(base);
   int8_t* cfg = base + sizeof_sharedv_aligned();
   T* hot = (T*)(cfg + k.smem_cfg_bytes);
-  X ex;
+  GroupExec<G, TC> ex;
   const long long slot = (long long)blockIdx.x * NG + g;
   T* ws = k.scratch + slot * k.ws_stride;
   init_trivial_slots(ex, k, ws);
@@ -1028,18 +1028,18 @@ __device__ void grouped_body(const KParams<T>& k) {
       __syncthreads();
     }
   }
-  tc_end(k, NG);
+  tc_end<T, TC>(k, NG);
 }
 
-template <class T>
+template <class T, bool TC>
 __global__ void __launch_bounds__(256, 2) vmc_kernel_grouped(const __grid_constant__ KParams<T> k) {
-  grouped_body<T, GroupExec<128>, 128>(k);
+  grouped_body<T, TC, 128>(k);
 }
 
 // Four chains per CTA of 512 threads (one CTA per SM).
-template <class T>
+template <class T, bool TC>
 __global__ void __launch_bounds__(512, 1) vmc_kernel_grouped4(const __grid_constant__ KParams<T> k) {
-  grouped_body<T, GroupExec<128>, 128>(k);
+  grouped_body<T, TC, 128>(k);
 }
 
 // Chains of several contexts (lattices of different sizes) in one persistent
@@ -1047,17 +1047,17 @@ __global__ void __launch_bounds__(512, 1) vmc_kernel_grouped4(const __grid_const
 // start[i+1] and is that context's chain g - start[i].  One chain per CTA;
 // the scratch arena has a slot of ws_stride (the largest of the contexts)
 // per CTA; dynamic shared memory is the largest of the contexts' needs.
-template <class T>
+template <class T, bool TC>
 __global__ void __launch_bounds__(256, 2)
     vmc_kernel_multi(const KParams<T>* __restrict__ ks, int n_ctx, const long long* __restrict__ start,
                      long long total, T* arena, long long ws_stride, unsigned long long* queue) {
   extern __shared__ __align__(16) int8_t dyn_smem[];
   __shared__ SharedV sv;
-  CtaExec ex;
+  CtaExecT<TC> ex;
   T* ws = arena + (long long)blockIdx.x * ws_stride;
   const int* tab = nullptr;
   int cur = -1;
-  tc_begin(ks[0], 1, dyn_smem, 0);
+  tc_begin<T, TC>(ks[0], 1, dyn_smem, 0);
   for (;;) {
     // the next chain of the launch's queue (contexts in the host's order,
     // the costliest first), taken when this CTA is free
@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(256, 2)
     }
     run_chain(ex, k, ws, sv, dyn_smem, (T*)(dyn_smem + k.smem_cfg_bytes), tab, (int)(gidx - start[i]));
   }
-  tc_end(ks[0], 1);
+  tc_end<T, TC>(ks[0], 1);
 }
 
 // The same with four chains per CTA of 512 threads (groups of 128, one CTA
@@ -1089,7 +1089,7 @@ __global__ void __launch_bounds__(256, 2)
 // (placement level 0) and do not keep lockstep; dynamic shared memory per
 // group: [SharedV][configuration of the largest context][tcgen05 staging]
 // [factorisation workspace] (offsets in the KParams, common to all contexts).
-template <class T>
+template <class T, bool TC>
 __global__ void __launch_bounds__(512, 1)
     vmc_kernel_multi4(const KParams<T>* __restrict__ ks, int n_ctx, const long long* __restrict__ start,
                       long long total, T* arena, long long ws_stride, long long group_bytes,
@@ -1098,11 +1098,11 @@ __global__ void __launch_bounds__(512, 1)
   constexpr int G = 128;
   const int g = threadIdx.x / G, NG = blockDim.x / G;
   if (threadIdx.x < 4) g_gemm_mode[threadIdx.x] = ks[0].gemm_mode;
-  tc_begin(ks[0], NG, dyn_smem, group_bytes);
+  tc_begin<T, TC>(ks[0], NG, dyn_smem, group_bytes);
   int8_t* base = dyn_smem + g * group_bytes;
   SharedV& sv = *reinterpret_cast<SharedV*>(base);
   int8_t* cfg = base + sizeof_sharedv_aligned();
-  GroupExec<G> ex;
+  GroupExec<G, TC> ex;
   const long long slot = (long long)blockIdx.x * NG + g;
   T* ws = arena + slot * ws_stride;
   int cur = -1;
@@ -1121,7 +1121,7 @@ __global__ void __launch_bounds__(512, 1)
     }
     run_chain(ex, k, ws, sv, cfg, (T*)(cfg + k.smem_cfg_bytes), k.tab, (int)(gidx - start[i]));
   }
-  tc_end(ks[0], NG);
+  tc_end<T, TC>(ks[0], NG);
 }
 
 }  // namespace gcf
