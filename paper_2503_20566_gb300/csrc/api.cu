@@ -917,9 +917,9 @@ gcf_status upload_params(gcf_ctx* c, const double* vals /* n_params or 2*n_param
 // instead of running on missing buffers.
 gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
   if (!c->sr.part) {
-    void** grp[12] = {(void**)&c->sr.obar, (void**)&c->sr.F, (void**)&c->sr.x, (void**)&c->sr.r,
+    void** grp[11] = {(void**)&c->sr.obar, (void**)&c->sr.F, (void**)&c->sr.x, (void**)&c->sr.r,
                       (void**)&c->sr.p, (void**)&c->sr.Ap, (void**)&c->sr.z, (void**)&c->sr.dinv,
-                      (void**)&c->sr.xf, (void**)&c->sr.tbar, (void**)&c->sr.scal, (void**)&c->sr.part};
+                      (void**)&c->sr.xf, (void**)&c->sr.scal, (void**)&c->sr.part};
     for (auto q : grp) {
       if (*q) cudaFree(*q);
       *q = nullptr;
@@ -930,7 +930,6 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
       if (!dalloc(v, sizeof(cdouble) * Np)) return fail(c, GCF_ENOMEM, "SR vectors");
     if (!dalloc(&c->sr.dinv, sizeof(double) * Np) ||
         !dalloc(&c->sr.xf, sizeof(float) * Np) ||
-        !dalloc(&c->sr.tbar, sizeof(cdouble)) ||
         !dalloc(&c->sr.scal, 32 * sizeof(double)) ||
         !dalloc(&c->sr.part, sizeof(cdouble) * kSumParts))
       return fail(c, GCF_ENOMEM, "SR vectors");
@@ -977,6 +976,8 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
     if (c->sr.perm) cudaFree(c->sr.perm);
     if (c->sr.osort) cudaFree(c->sr.osort);
     if (c->sr.coef_f) cudaFree(c->sr.coef_f);
+    if (c->sr.count) cudaFree(c->sr.count);
+    c->sr.count = nullptr;
     c->sr.t = c->sr.coef = nullptr;
     c->sr.perm = nullptr;
     c->sr.osort = nullptr;
@@ -987,6 +988,9 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
         !dalloc(&c->sr.coef_f, sizeof(float) * Ns) ||
         !dalloc(&c->sr.perm, sizeof(int) * Ns * c->n_s) ||
         !dalloc(&c->sr.osort, c->sbytes * (size_t)Ns * c->sr_sum_bs))
+      return fail(c, GCF_ENOMEM, "SR sample vectors");
+    // the chunked sort's table, where it is small beside the rest (else the sort that needs none)
+    if (c->sr.maxnb <= 128 && !dalloc(&c->sr.count, sizeof(int) * (size_t)c->n_s * c->sr.maxnb * ((Ns + 1023) / 1024)))
       return fail(c, GCF_ENOMEM, "SR sample vectors");
     c->sr_ns_cap = Ns;
   }
@@ -1096,7 +1100,7 @@ void gcf_destroy(gcf_ctx* c) {
   if (!c) return;
   void* ptrs[] = {c->d_params, c->d_Q, c->d_voff, c->d_vbs, c->d_vnb, c->d_tables, c->d_status,
                   c->d_scratch, c->sr.obar, c->sr.F, c->sr.x, c->sr.r, c->sr.p, c->sr.Ap, c->sr.z, c->sr.dinv,
-                  c->sr.t, c->sr.coef, c->sr.chain_mean, c->sr.tbar, c->sr.scal, c->sr.perm, c->sr.seg,
+                  c->sr.t, c->sr.coef, c->sr.chain_mean, c->sr.scal, c->sr.perm, c->sr.seg, c->sr.count,
                   c->sr.pbs, c->sr.osort, c->sr.xf, c->sr.coef_f, c->sr.part,
                   c->sr.seg_v, c->sr.seg_b, c->d_cfg, c->d_e,
                   c->d_la, c->d_ph, c->d_bid, c->d_O, c->d_acc, c->vjp_bid, c->vjp_O, c->vjp_coef,

@@ -22,30 +22,6 @@ __device__ inline cdouble to_cd(T v) {
   return {(double)re(v), (double)im(v)};
 }
 
-// t_s = sum_v sum_e O[s][v][e] * x[off(v, bid) + e]; one warp per sample.
-template <class T>
-__global__ void k_gather_dot(SrGeom g, const int* bids, const T* O, const cdouble* x, cdouble* t) {
-  const int lane = threadIdx.x & 31;
-  const long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (s >= g.Ns) return;
-  double ar = 0.0, ai = 0.0;
-  for (int v = 0; v < g.n_s; ++v) {
-    const int bid = bids[s * g.n_s + v];
-    const int bs = g.vbs[v];
-    const long long base = g.voff[v] + (long long)bid * bs;
-    const T* o = O + (s * g.n_s + v) * (long long)g.D4;
-    for (int e = lane; e < bs; e += 32) {
-      const cdouble a = to_cd(o[e]);
-      const cdouble b = x[base + e];
-      ar += a.x * b.x - a.y * b.y;
-      ai += a.x * b.y + a.y * b.x;
-    }
-  }
-  ar = warp_sum(ar);
-  ai = warp_sum(ai);
-  if (lane == 0) t[s] = {ar, ai};
-}
-
 // out[off(v,bid)+e] += sum_s coef_s * conj?(O[s][v][e]) for one vertex per
 // blockIdx.y and a chunk of samples per blockIdx.x; block-local accumulation
 // in shared memory (all blocks of the vertex), flushed with global atomics.
@@ -94,6 +70,19 @@ __global__ void k_chain_means(const double* e, int n_per_chain, cdouble* chain_m
   if (threadIdx.x == 0) chain_mean[c] = {r / n_per_chain, i / n_per_chain};
 }
 
+// the same for chains of few samples, a thread per chain (a block per chain of
+// one sample each took 486 us for 65536 chains, this 3)
+__global__ void k_chain_means_short(const double* e, int n_per_chain, long long n_chains, cdouble* chain_mean) {
+  const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n_chains) return;
+  double r = 0.0, i = 0.0;
+  for (int s = 0; s < n_per_chain; ++s) {
+    r += e[2 * (c * n_per_chain + s)];
+    i += e[2 * (c * n_per_chain + s) + 1];
+  }
+  chain_mean[c] = {r / n_per_chain, i / n_per_chain};
+}
+
 // mean and std error over m values (single block); out[0..2] = Re, Im, err
 __global__ void k_mean_err(const cdouble* v, int m, double* out) {
   __shared__ double red[64];
@@ -118,23 +107,8 @@ __global__ void k_f_coef(const double* e, long long Ns, const double* emean, cdo
   coef[s] = {(e[2 * s] - emean[0]) / (double)Ns, (e[2 * s + 1] - emean[1]) / (double)Ns};
 }
 
-// coef_s = (t_s - tbar) / Ns where tbar = mean t
-__global__ void k_center(cdouble* t, long long Ns, const cdouble* tbar) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= Ns) return;
-  t[s] = {(t[s].x - tbar->x) / (double)Ns, (t[s].y - tbar->y) / (double)Ns};
-}
-
-__global__ void k_sum_c(const cdouble* v, long long n, cdouble* out, double scale_) {
-  __shared__ double red[64];
-  double r = 0.0, i = 0.0;
-  for (long long k = threadIdx.x; k < n; k += blockDim.x) { r += v[k].x; i += v[k].y; }
-  block_sum2(r, i, red);
-  if (threadIdx.x == 0) *out = {r * scale_, i * scale_};
-}
-
 // First stage of a deterministic sum over many blocks: block b writes the sum
-// of its grid-stride share to part[b]; k_sum_c over part[] finishes it.
+// of its grid-stride share to part[b]; k_center finishes it.
 __global__ void k_sum_c_part(const cdouble* v, long long n, cdouble* part) {
   __shared__ double red[64];
   double r = 0.0, i = 0.0;
@@ -145,6 +119,22 @@ __global__ void k_sum_c_part(const cdouble* v, long long n, cdouble* part) {
   }
   block_sum2(r, i, red);
   if (threadIdx.x == 0) part[blockIdx.x] = {r, i};
+}
+
+// t_s <- (t_s - tbar) / Ns with tbar the mean of t: every block sums the parts
+// of k_sum_c_part for itself.  coef_f, if set: the FP32 copy of the real parts.
+__global__ void k_center(cdouble* t, long long Ns, const cdouble* part, int n_part, float* coef_f) {
+  __shared__ double red[64];
+  double r = 0.0, i = 0.0;
+  for (int k = threadIdx.x; k < n_part; k += blockDim.x) { r += part[k].x; i += part[k].y; }
+  block_sum2(r, i, red);
+  r /= (double)Ns;
+  i /= (double)Ns;
+  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= Ns) return;
+  const cdouble v = {(t[s].x - r) / (double)Ns, (t[s].y - i) / (double)Ns};
+  t[s] = v;
+  if (coef_f) coef_f[s] = (float)v.x;
 }
 
 // FP32 copy of the real parts of a vector.  The FP32-storage kernels form
@@ -168,30 +158,58 @@ __global__ void k_dot(const cdouble* a, const cdouble* b, long long n, double* o
   if (threadIdx.x == 0) { atomicAdd(&out[0], r); atomicAdd(&out[1], i); }
 }
 
-// y = y + lambda x (the diagonal shift)
-__global__ void k_axpy_real(cdouble* y, const cdouble* x, double a, long long n) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) { y[k].x += a * x[k].x; y[k].y += a * x[k].y; }
+// Ap += shift p, then *out += Re <p, Ap> (S is Hermitian)
+__global__ void k_shift_dot(cdouble* Ap, const cdouble* p, double shift, long long n, double* out) {
+  __shared__ double red[64];
+  double r = 0.0;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+       k += (long long)gridDim.x * blockDim.x) {
+    const cdouble q = p[k];
+    cdouble a = Ap[k];
+    a.x += shift * q.x;
+    a.y += shift * q.y;
+    Ap[k] = a;
+    r += q.x * a.x + q.y * a.y;
+  }
+  r = block_sum(r, red);
+  if (threadIdx.x == 0) atomicAdd(out, r);
 }
 
-// CG vector update: x += alpha p; r -= alpha Ap; alpha = rz / pAp (real)
-__global__ void k_cg_xr(cdouble* x, cdouble* r, const cdouble* p, const cdouble* Ap,
-                        const double* sc, long long n) {
-  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const double alpha = sc[0] / sc[2];
-  x[k].x += alpha * p[k].x; x[k].y += alpha * p[k].y;
-  r[k].x -= alpha * Ap[k].x; r[k].y -= alpha * Ap[k].y;
+// x += alpha p, r -= alpha Ap with alpha = rz / pAp (real), z = M^-1 r;
+// *rz_new += <r, z>, *rr += <r, r>
+__global__ void k_cg_xr(cdouble* x, cdouble* r, cdouble* z, const cdouble* p, const cdouble* Ap, const double* dinv,
+                        const double* rz, const double* pAp, double* rz_new, double* rr, long long n) {
+  __shared__ double red[64];
+  const double alpha = *rz / *pAp;
+  double sz = 0.0, sr = 0.0;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
+       k += (long long)gridDim.x * blockDim.x) {
+    x[k].x += alpha * p[k].x;
+    x[k].y += alpha * p[k].y;
+    const cdouble v = {r[k].x - alpha * Ap[k].x, r[k].y - alpha * Ap[k].y};
+    const double d = dinv[k];
+    r[k] = v;
+    z[k] = {d * v.x, d * v.y};
+    const double a = v.x * v.x + v.y * v.y;
+    sr += a;
+    sz += d * a;
+  }
+  block_sum2(sz, sr, red);
+  if (threadIdx.x == 0) {
+    atomicAdd(rz_new, sz);
+    atomicAdd(rr, sr);
+  }
 }
 
-// p = z + beta p, beta = rz_new / rz_old (z = M^-1 r; z = r without
-// preconditioning)
-__global__ void k_cg_p(cdouble* p, const cdouble* z, const double* sc, long long n) {
+// p = z + beta p, beta = rz_new / rz_old; xf, if set: the FP32 copy of its real parts
+__global__ void k_cg_p(cdouble* p, const cdouble* z, const double* rz_new, const double* rz_old, float* xf,
+                       long long n) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  const double beta = sc[4] / sc[0];
-  p[k].x = z[k].x + beta * p[k].x;
-  p[k].y = z[k].y + beta * p[k].y;
+  const double beta = *rz_new / *rz_old;
+  const cdouble v = {z[k].x + beta * p[k].x, z[k].y + beta * p[k].y};
+  p[k] = v;
+  if (xf) xf[k] = (float)v.x;
 }
 
 // params += c * x  (c complex); real storage takes the real part
@@ -246,6 +264,90 @@ __global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm,
   if (threadIdx.x == 0) seg[v * (maxnb + 1) + nb] = base_s;
 }
 
+// The same order from three passes over chunks of 1024 samples, for at most
+// kSortBlocks blocks a vertex (one CTA per vertex walks all samples once per
+// block above: 905 us at 65536 samples on 8x8, this 40).  count: [vertex][block]
+// [chunk], turned from counts into starts by the middle pass.
+constexpr int kSortBlocks = 128;
+__device__ __forceinline__ int sort_rank(const int* bids, const SrGeom& g, int v, int nb, int* wcnt, int& b, bool& in) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long s = (long long)blockIdx.x * 1024 + threadIdx.x;
+  in = s < g.Ns;
+  b = in ? bids[s * g.n_s + v] : -1;
+  for (int i = threadIdx.x; i < 32 * nb; i += 1024) wcnt[i] = 0;
+  __syncthreads();
+  const unsigned m = __match_any_sync(0xffffffffu, b);
+  const int before = __popc(m & ((1u << lane) - 1u));
+  if (in && before == 0) wcnt[wid * nb + b] = __popc(m);
+  __syncthreads();
+  return before;
+}
+__global__ void k_sort_count(SrGeom g, const int* bids, int maxnb, int n_chunk, int* count) {
+  extern __shared__ int wcnt[];
+  const int v = blockIdx.y, nb = g.vnb[v];
+  int b;
+  bool in;
+  sort_rank(bids, g, v, nb, wcnt, b, in);
+  for (int i = threadIdx.x; i < nb; i += 1024) {
+    int t = 0;
+    for (int w = 0; w < 32; ++w) t += wcnt[w * nb + i];
+    count[((long long)v * maxnb + i) * n_chunk + blockIdx.x] = t;
+  }
+}
+__global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* seg) {
+  __shared__ int tot[kSortBlocks + 1];
+  const int v = blockIdx.x, nb = g.vnb[v], lane = threadIdx.x & 31;
+  int* cv = count + (long long)v * maxnb * n_chunk;
+  for (int b = threadIdx.x >> 5; b < nb; b += blockDim.x >> 5) {
+    int t = 0;
+    for (int i = lane; i < n_chunk; i += 32) t += cv[b * n_chunk + i];
+    t = warp_sum(t);
+    if (lane == 0) tot[b] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int acc = 0;
+    for (int b = 0; b < nb; ++b) {
+      const int t = tot[b];
+      tot[b] = acc;
+      seg[v * (maxnb + 1) + b] = acc;
+      acc += t;
+    }
+    seg[v * (maxnb + 1) + nb] = acc;
+  }
+  __syncthreads();
+  for (int b = threadIdx.x >> 5; b < nb; b += blockDim.x >> 5) {
+    int base = tot[b];
+    for (int i0 = 0; i0 < n_chunk; i0 += 32) {
+      const int i = i0 + lane, c = i < n_chunk ? cv[b * n_chunk + i] : 0;
+      int inc = c;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+      }
+      if (i < n_chunk) cv[b * n_chunk + i] = base + inc - c;
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+  }
+}
+__global__ void k_sort_place(SrGeom g, const int* bids, int maxnb, int n_chunk, const int* count, int* perm) {
+  extern __shared__ int wcnt[];
+  const int v = blockIdx.y, nb = g.vnb[v];
+  int b;
+  bool in;
+  const int before = sort_rank(bids, g, v, nb, wcnt, b, in);
+  for (int i = threadIdx.x; i < nb; i += 1024) {
+    int t = count[((long long)v * maxnb + i) * n_chunk + blockIdx.x];
+    for (int w = 0; w < 32; ++w) {
+      const int c = wcnt[w * nb + i];
+      wcnt[w * nb + i] = t;
+      t += c;
+    }
+  }
+  __syncthreads();
+  if (in) perm[(long long)v * g.Ns + wcnt[(threadIdx.x >> 5) * nb + b] + before] = blockIdx.x * 1024 + threadIdx.x;
+}
+
 // storage-precision accumulator type: FP32 forms accumulate short partial
 // sums in float before adding them into FP64
 template <class T> struct PartialOf { using type = double; };
@@ -290,20 +392,25 @@ __global__ void k_gather2(SrGeom g, const int* bids, const T* O, const cdouble* 
 // The same product with each sample's O row (n_s x D4 storage scalars,
 // contiguous) read by the whole warp in 16-byte vectors; needs D4 a multiple
 // of VE = 16 / sizeof(T).  Per-vector partials in the storage precision,
-// then FP64.
-template <class T, bool CPLX>
+// then FP64.  BLK: by a block of 256 instead of a warp, for few samples (1024
+// warps leave the chip idle: 74 us at 1024 complex samples of 16x16, D_k = 2;
+// the floor of 34 MB is 5).
+constexpr long long kBlockGatherBelow = 16384;  // samples: 152 SMs x 64 warps hold about 10000
+template <class T, bool CPLX, bool BLK>
 __global__ void k_gather_vec(SrGeom g, const int* bids, const T* O, const cdouble* x, cdouble* t) {
   using P = typename PartialOf<T>::type;
   constexpr int VE = 16 / (int)sizeof(T);
-  const int lane = threadIdx.x & 31;
-  const long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  __shared__ double red[64];
+  const int lane = BLK ? threadIdx.x : threadIdx.x & 31;
+  constexpr int STEP = BLK ? 256 : 32;
+  const long long s = BLK ? (long long)blockIdx.x : ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (s >= g.Ns) return;
   const int nvec = g.n_s * g.D4 / VE;
   const float4* row = reinterpret_cast<const float4*>(O + s * g.n_s * (long long)g.D4);
   const int* brow = bids + s * g.n_s;
   double ar = 0.0, ai = 0.0;
-#pragma unroll 2
-  for (int j = lane; j < nvec; j += 32) {
+#pragma unroll 4
+  for (int j = lane; j < nvec; j += STEP) {
     const int el = j * VE, v = el / g.D4, e0 = el - v * g.D4;
     const int bs = g.vbs[v];
     if (e0 >= bs) continue;
@@ -326,25 +433,33 @@ __global__ void k_gather_vec(SrGeom g, const int* bids, const T* O, const cdoubl
     ar += (double)pr;
     if (CPLX) ai += (double)pi;
   }
-  ar = warp_sum(ar);
-  if (CPLX) ai = warp_sum(ai);
+  if constexpr (BLK) {
+    block_sum2(ar, ai, red);
+  } else {
+    ar = warp_sum(ar);
+    if (CPLX) ai = warp_sum(ai);
+  }
   if (lane == 0) t[s] = {ar, CPLX ? ai : 0.0};
 }
 
 // k_gather_vec for real FP32 storage whose block sizes (hence vertex offsets)
 // are multiples of 4, with D4 = 2^d4_shift: the direction x comes as its FP32
 // copy xf and is read in 16-byte quads like O.  Same products, same order.
+// Eight quads in flight a lane (two: 89 us at 65536 samples of 8x8).
+template <bool BLK>
 __global__ void k_gather_f4(SrGeom g, const int* bids, const float* O, const float* xf, int d4_shift,
                             cdouble* t) {
-  const int lane = threadIdx.x & 31;
-  const long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  __shared__ double red[64];
+  const int lane = BLK ? threadIdx.x : threadIdx.x & 31;
+  constexpr int STEP = BLK ? 256 : 32;
+  const long long s = BLK ? (long long)blockIdx.x : ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (s >= g.Ns) return;
   const int nvec = (g.n_s * g.D4) >> 2;
   const float4* row = reinterpret_cast<const float4*>(O + s * g.n_s * (long long)g.D4);
   const int* brow = bids + s * g.n_s;
   double ar = 0.0;
-#pragma unroll 2
-  for (int j = lane; j < nvec; j += 32) {
+#pragma unroll 8
+  for (int j = lane; j < nvec; j += STEP) {
     const int el = j << 2, v = el >> d4_shift, e0 = el - (v << d4_shift);
     const int bs = g.vbs[v];
     if (e0 >= bs) continue;
@@ -357,7 +472,7 @@ __global__ void k_gather_f4(SrGeom g, const int* bids, const float* O, const flo
     pr += o.w * xq.w;
     ar += (double)pr;
   }
-  ar = warp_sum(ar);
+  ar = BLK ? block_sum(ar, red) : warp_sum(ar);
   if (lane == 0) t[s] = {ar, 0.0};
 }
 
@@ -374,6 +489,20 @@ __global__ void k_permute_O(SrGeom g, const int* perm, const long long* pbs, con
     const long long q = i / bs;
     const int e = (int)(i - q * bs);
     dst[i] = O[((long long)pv[q] * g.n_s + v) * g.D4 + e];
+  }
+}
+
+// k_permute_O for real FP32 storage whose block sizes are multiples of 4, in
+// 16-byte quads and 32-bit indexes (Ns * bs < 2^31).
+__global__ void k_permute_f4(SrGeom g, const int* perm, const long long* pbs, const float* O, float* osort) {
+  const int v = blockIdx.y;
+  const int nq = g.vbs[v] >> 2, n = (int)g.Ns * nq;
+  const int* pv = perm + (long long)v * g.Ns;
+  float4* dst = reinterpret_cast<float4*>(osort + g.Ns * pbs[v]);
+#pragma unroll 4
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int q = i / nq, e = i - q * nq;
+    dst[i] = *reinterpret_cast<const float4*>(O + ((long long)pv[q] * g.n_s + v) * g.D4 + 4 * e);
   }
 }
 
@@ -447,7 +576,63 @@ __global__ void k_scatter_sorted(SrGeom g, const int* perm, const int* seg, int 
   }
 }
 
-// Real FP32 storage with bs a multiple of 4: each thread takes a 16-byte
+// k_scatter_sorted with a warp per segment, for short segments of blocks of at
+// most 32 entries: lanes take 32 / bs rows at a time (a CTA per segment of 38
+// rows: 80 us at 1024 complex samples of 16x16 Z3).
+template <class T, bool CONJ, bool CPLX, bool SQ>
+__global__ void k_scatter_warp(SrGeom g, const int* perm, const int* seg, int maxnb, int n_seg, const T* osort,
+                               const long long* pbs, const cdouble* coef, cdouble* out, const int* seg_v,
+                               const int* seg_b) {
+  using P = typename PartialOf<T>::type;
+  const int lane = threadIdx.x & 31;
+  const int sid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (sid >= n_seg) return;
+  const int v = seg_v[sid], b = seg_b[sid];
+  const int bs = g.vbs[v], rpw = 32 / bs;
+  const int s0 = seg[v * (maxnb + 1) + b], s1 = seg[v * (maxnb + 1) + b + 1];
+  if (s0 >= s1) return;
+  const int* pv = perm + (long long)v * g.Ns;
+  const T* rows = osort + g.Ns * pbs[v];
+  const int rr = lane / bs, e = lane - rr * bs;
+  double ar = 0.0, ai = 0.0;
+  if (rr < rpw) {
+    for (int q0 = s0 + rr; q0 < s1; q0 += 32 * rpw) {  // FP32 partial sums over 32 rows
+      P pr = P(0), pi = P(0);
+#pragma unroll 8
+      for (int i = 0; i < 32; ++i) {
+        const int q = q0 + i * rpw;
+        if (q >= s1) break;
+        const T ov = rows[(long long)q * bs + e];
+        const cdouble c = coef[pv[q]];
+        P orr = (P)re(ov), oi = CONJ ? -(P)im(ov) : (P)im(ov);
+        if (SQ) {
+          orr = orr * orr + oi * oi;
+          oi = P(0);
+        }
+        if (CPLX && !SQ) {
+          pr += (P)c.x * orr - (P)c.y * oi;
+          pi += (P)c.x * oi + (P)c.y * orr;
+        } else {
+          pr += (P)c.x * orr;
+        }
+      }
+      ar += (double)pr;
+      ai += (double)pi;
+    }
+  }
+  double sr = ar, si = ai;
+  for (int r = 1; r < rpw; ++r) {
+    sr += __shfl_sync(0xffffffffu, ar, (lane + r * bs) & 31);
+    if (CPLX) si += __shfl_sync(0xffffffffu, ai, (lane + r * bs) & 31);
+  }
+  if (lane < bs) {
+    cdouble* dst = out + g.voff[v] + (long long)b * bs + lane;
+    atomicAdd(&dst->x, sr);
+    if (CPLX) atomicAdd(&dst->y, si);
+  }
+}
+
+// Real FP32 storage with bs = 4, 8 or 16 (D_k = 2): each thread takes a 16-byte
 // quad (4 entries) of a row, and the coefficients come as the FP32 copy of
 // their real parts (the values the products use); otherwise as
 // k_scatter_sorted.
@@ -455,7 +640,7 @@ template <bool SQ>
 __global__ void k_scatter_sorted_f4(SrGeom g, const int* perm, const int* seg, int maxnb, int split,
                                     const float* osort, const long long* pbs, const float* coef, cdouble* out,
                                     const int* seg_v, const int* seg_b) {
-  __shared__ double red[256 * 4];
+  __shared__ double red[8 * 16];
   const int sid = blockIdx.x / split, part = blockIdx.x - (blockIdx.x / split) * split;
   const int v = seg_v[sid], b = seg_b[sid];
   const int bs = g.vbs[v], nq = bs >> 2;
@@ -469,35 +654,44 @@ __global__ void k_scatter_sorted_f4(SrGeom g, const int* perm, const int* seg, i
   const int rps = max(1, (int)blockDim.x / nq);  // rows per step
   const int qi = threadIdx.x % nq, rr = threadIdx.x / nq;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  if (rr < rps) {
-    int cnt = 0;
+  // FP32 partial sums over 32 rows; eight rows in flight (their coefficients
+  // come through perm; two in flight: 132 us at 65536 samples of 8x8)
+  for (int q0 = s_begin + rr; q0 < s_end; q0 += 32 * rps) {
     float part4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-    for (int q = s_begin + rr; q < s_end; q += rps) {
-      const float4 o = *reinterpret_cast<const float4*>(rows + (long long)q * bs + 4 * qi);
-      const float c = coef[pv[q]];
-      if (SQ) {
-        part4[0] += c * o.x * o.x; part4[1] += c * o.y * o.y;
-        part4[2] += c * o.z * o.z; part4[3] += c * o.w * o.w;
-      } else {
-        part4[0] += c * o.x; part4[1] += c * o.y; part4[2] += c * o.z; part4[3] += c * o.w;
-      }
-      if (++cnt == 32) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { acc[i] += (double)part4[i]; part4[i] = 0.f; }
-        cnt = 0;
+    for (int i0 = 0; i0 < 32; i0 += 8) {
+      float c[8];
+      float4 o[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int q = q0 + (i0 + i) * rps;
+        const bool in = q < s_end;
+        c[i] = in ? coef[pv[q]] : 0.f;
+        o[i] = in ? *reinterpret_cast<const float4*>(rows + (long long)q * bs + 4 * qi) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (SQ) {
+          part4[0] += c[i] * o[i].x * o[i].x; part4[1] += c[i] * o[i].y * o[i].y;
+          part4[2] += c[i] * o[i].z * o[i].z; part4[3] += c[i] * o[i].w * o[i].w;
+        } else {
+          part4[0] += c[i] * o[i].x; part4[1] += c[i] * o[i].y; part4[2] += c[i] * o[i].z; part4[3] += c[i] * o[i].w;
+        }
       }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[i] += (double)part4[i];
   }
+  // lanes of the same quad (nq = 1, 2 or 4 apart), then the eight warps
 #pragma unroll
-  for (int i = 0; i < 4; ++i) red[4 * threadIdx.x + i] = acc[i];
+  for (int i = 0; i < 4; ++i) {
+    for (int o = nq; o < 32; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+    if ((threadIdx.x & 31) < nq) red[(threadIdx.x >> 5) * 16 + 4 * (threadIdx.x & 31) + i] = acc[i];
+  }
   __syncthreads();
   if (threadIdx.x < bs) {
-    const int q4 = threadIdx.x >> 2, i = threadIdx.x & 3;
     double sr = 0.0;
-    for (int r = 0; r < rps; ++r) sr += red[4 * (r * nq + q4) + i];
+    for (int w = 0; w < 8; ++w) sr += red[w * 16 + threadIdx.x];
     atomicAdd(&(out + g.voff[v] + (long long)b * bs + threadIdx.x)->x, sr);
   }
 }
@@ -511,8 +705,6 @@ __global__ void k_e_to_c(const double* e, long long n, cdouble* v) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) v[k] = {e[2 * k], e[2 * k + 1]};
 }
-
-__global__ void k_copy_scalar(double* sc) { sc[0] = sc[4]; sc[1] = sc[5]; }
 
 // Jacobi preconditioner of S + shift: diag(S)_m = <|O_m|^2> - |<O_m>|^2
 // (clamped at 0 against rounding); dinv = 1 / (diag + shift).
@@ -540,7 +732,8 @@ static inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
 template <class T>
 static cudaError_t scatter(const SrGeom& g, const SrWork& w, const T* O, const cdouble* coef,
-                           cdouble* out, bool conj, cudaStream_t st, long long* launches, bool sq = false) {
+                           cdouble* out, bool conj, cudaStream_t st, long long* launches, bool sq = false,
+                           bool have_f = false) {
   constexpr bool C = Traits<T>::cplx;
   // about 2048 samples per CTA: the average segment holds Ns * n_s / n_seg
   const long long per_seg = g.Ns * g.n_s / std::max(1, w.n_seg);
@@ -550,16 +743,33 @@ static cudaError_t scatter(const SrGeom& g, const SrWork& w, const T* O, const c
   (void)O;
   if constexpr (std::is_same<T, float>::value) {
     if (w.all_bs4) {
-      k_real_to_f32<<<nblk(g.Ns, 256), 256, 0, st>>>(coef, g.Ns, w.coef_f);
+      if (!have_f) {
+        k_real_to_f32<<<nblk(g.Ns, 256), 256, 0, st>>>(coef, g.Ns, w.coef_f);
+        ++*launches;
+      }
       if (sq)
         k_scatter_sorted_f4<true><<<grid, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, split, os, w.pbs, w.coef_f,
                                                          out, w.seg_v, w.seg_b);
       else
         k_scatter_sorted_f4<false><<<grid, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, split, os, w.pbs, w.coef_f,
                                                           out, w.seg_v, w.seg_b);
-      *launches += 2;
+      ++*launches;
       return cudaGetLastError();
     }
+  }
+  if (g.D4 <= 32 && per_seg < 256) {
+    const int blocks = nblk((long long)w.n_seg * 32, 256);
+    if (sq)
+      k_scatter_warp<T, false, C, true><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
+                                                                out, w.seg_v, w.seg_b);
+    else if (conj)
+      k_scatter_warp<T, true, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
+                                                                out, w.seg_v, w.seg_b);
+    else
+      k_scatter_warp<T, false, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
+                                                                 out, w.seg_v, w.seg_b);
+    ++*launches;
+    return cudaGetLastError();
   }
   if (sq)
     k_scatter_sorted<T, false, C, true><<<grid, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, split, os, w.pbs, coef,
@@ -605,7 +815,10 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   } while (0)
   // energy mean and error bar (over chain means, or over samples for one chain)
   if (n_chains > 1) {
-    k_chain_means<<<n_chains, 256, 0, st>>>(e_loc, (int)(Ns / n_chains), w.chain_mean);
+    if (Ns / n_chains < 64)
+      k_chain_means_short<<<nblk(n_chains, 256), 256, 0, st>>>(e_loc, (int)(Ns / n_chains), n_chains, w.chain_mean);
+    else
+      k_chain_means<<<n_chains, 256, 0, st>>>(e_loc, (int)(Ns / n_chains), w.chain_mean);
     ++*launches;
     k_mean_err<<<1, 1024, 0, st>>>(w.chain_mean, n_chains, w.scal);
   } else {
@@ -616,12 +829,27 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   ++*launches;
   CK(cudaGetLastError());
   // samples grouped by (vertex, block) for the atomic-free scatter
-  k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg);
-  ++*launches;
+  if (w.count) {
+    const int n_chunk = nblk(Ns, 1024);
+    const dim3 grid((unsigned)n_chunk, (unsigned)g.n_s);
+    const size_t smem = sizeof(int) * 32 * w.maxnb;
+    k_sort_count<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count);
+    k_sort_scan<<<g.n_s, 256, 0, st>>>(g, w.maxnb, n_chunk, w.count, w.seg);
+    k_sort_place<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count, w.perm);
+    *launches += 3;
+  } else {
+    k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg);
+    ++*launches;
+  }
   // O in segment order, streamed by every scatter of this step
   {
     dim3 grid((unsigned)std::min<long long>(1024, (Ns * 16 + 255) / 256), (unsigned)g.n_s);
-    k_permute_O<T><<<grid, 256, 0, st>>>(g, w.perm, w.pbs, O, (T*)w.osort);
+    bool quads = false;
+    if constexpr (std::is_same<T, float>::value) {
+      quads = vec_ok && w.all_bs4 && Ns * g.D4 < (1LL << 31);
+      if (quads) k_permute_f4<<<grid, 256, 0, st>>>(g, w.perm, w.pbs, O, (float*)w.osort);
+    }
+    if (!quads) k_permute_O<T><<<grid, 256, 0, st>>>(g, w.perm, w.pbs, O, (T*)w.osort);
     ++*launches;
   }
   // Obar = (1/Ns) sum_s O_s
@@ -651,7 +879,8 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   }
   ++*launches;
   // preconditioned CG: x = 0, r = F, z = M^-1 r, p = z
-  double* sc = w.scal + 8;  // sc[0..1] rz, sc[2..3] pAp, sc[4..5] rz_new, sc[6..7] rr
+  double* sc = w.scal + 8;  // sc[0..1] rz, sc[2..3] pAp, sc[4..5] rz_new, sc[6..7] rr (imaginary parts unused)
+  double *rz = sc, *rz_new = sc + 4;  // swapped every iteration
   CK(cudaMemsetAsync(w.x, 0, sizeof(cdouble) * Np, st));
   CK(cudaMemcpyAsync(w.r, w.F, sizeof(cdouble) * Np, cudaMemcpyDeviceToDevice, st));
   k_precond<<<nblk(Np, 256), 256, 0, st>>>(w.z, w.r, w.dinv, Np);
@@ -668,44 +897,40 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   double rr = rr0;
   int it = 0;
   bool converged = !(fnorm > 0.0);
+  bool quad = false;
+  if constexpr (std::is_same<T, float>::value) quad = vec_ok && w.all_bs4 && d4_shift >= 2;
+  const bool blk = Ns < kBlockGatherBelow;
+  const int vgrid = (int)std::min<long long>(nblk(Np, 256), 1024);
+  if (quad && !converged && max_iter > 0) {
+    k_real_to_f32<<<nblk(Np, 256), 256, 0, st>>>(w.p, Np, w.xf);
+    ++*launches;
+  }
   while (!converged && it < max_iter) {
     // Ap = S p + shift p
-    bool quad = false;
-    if constexpr (std::is_same<T, float>::value) {
-      if (vec_ok && w.all_bs4 && d4_shift >= 2) {
-        k_real_to_f32<<<nblk(Np, 256), 256, 0, st>>>(w.p, Np, w.xf);
-        k_gather_f4<<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.xf, d4_shift, w.t);
-        *launches += 2;
-        quad = true;
+    if (quad) {
+      if constexpr (std::is_same<T, float>::value) {
+        if (blk) k_gather_f4<true><<<(unsigned)Ns, 256, 0, st>>>(g, bids, O, w.xf, d4_shift, w.t);
+        else k_gather_f4<false><<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.xf, d4_shift, w.t);
       }
-    }
-    if (!quad) {
-      if (vec_ok)
-        k_gather_vec<T, Traits<T>::cplx><<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.p, w.t);
-      else
-        k_gather2<T, Traits<T>::cplx><<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.p, w.t);
-      ++*launches;
+    } else if (vec_ok) {
+      if (blk) k_gather_vec<T, Traits<T>::cplx, true><<<(unsigned)Ns, 256, 0, st>>>(g, bids, O, w.p, w.t);
+      else k_gather_vec<T, Traits<T>::cplx, false><<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.p, w.t);
+    } else {
+      k_gather2<T, Traits<T>::cplx><<<nblk(Ns * 32, 256), 256, 0, st>>>(g, bids, O, w.p, w.t);
     }
     k_sum_c_part<<<kSumParts, 256, 0, st>>>(w.t, Ns, w.part);
-    k_sum_c<<<1, 1024, 0, st>>>(w.part, kSumParts, w.tbar, 1.0 / (double)Ns);
-    *launches += 2;
-    k_center<<<nblk(Ns, 256), 256, 0, st>>>(w.t, Ns, w.tbar);
-    ++*launches;
+    k_center<<<nblk(Ns, 256), 256, 0, st>>>(w.t, Ns, w.part, kSumParts, quad ? w.coef_f : nullptr);
+    *launches += 3;
     CK(cudaMemsetAsync(w.Ap, 0, sizeof(cdouble) * Np, st));
-    CK(scatter<T>(g, w, O, w.t, w.Ap, true, st, launches));
-    k_axpy_real<<<nblk(Np, 256), 256, 0, st>>>(w.Ap, w.p, shift, Np);
-    ++*launches;
-    CK(dot<T>(w.p, w.Ap, Np, sc + 2, st, launches));
-    k_cg_xr<<<nblk(Np, 256), 256, 0, st>>>(w.x, w.r, w.p, w.Ap, sc, Np);
-    ++*launches;
-    k_precond<<<nblk(Np, 256), 256, 0, st>>>(w.z, w.r, w.dinv, Np);
-    ++*launches;
-    CK(dot<T>(w.r, w.z, Np, sc + 4, st, launches));
-    CK(dot<T>(w.r, w.r, Np, sc + 6, st, launches));
-    k_cg_p<<<nblk(Np, 256), 256, 0, st>>>(w.p, w.z, sc, Np);
-    ++*launches;
-    k_copy_scalar<<<1, 1, 0, st>>>(sc);
-    ++*launches;
+    CK(cudaMemsetAsync(sc + 2, 0, 2 * sizeof(double), st));
+    CK(cudaMemsetAsync(rz_new, 0, sizeof(double), st));
+    CK(cudaMemsetAsync(sc + 6, 0, sizeof(double), st));
+    CK(scatter<T>(g, w, O, w.t, w.Ap, true, st, launches, false, quad));
+    k_shift_dot<<<vgrid, 256, 0, st>>>(w.Ap, w.p, shift, Np, sc + 2);
+    k_cg_xr<<<vgrid, 256, 0, st>>>(w.x, w.r, w.z, w.p, w.Ap, w.dinv, rz, sc + 2, rz_new, sc + 6, Np);
+    k_cg_p<<<nblk(Np, 256), 256, 0, st>>>(w.p, w.z, rz_new, rz, quad ? w.xf : nullptr, Np);
+    *launches += 3;
+    std::swap(rz, rz_new);
     double rn;
     CK(cudaMemcpyAsync(&rn, sc + 6, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));

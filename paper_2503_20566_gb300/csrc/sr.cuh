@@ -27,11 +27,11 @@ struct SrWork {
   double* dinv;                        // [Np] inverse Jacobi preconditioner
   cdouble *t, *coef;                   // [Ns]
   cdouble *chain_mean;                 // [n_chains]
-  cdouble *tbar;                       // [1]
   double* scal;                        // [16] device scalars
   // sample order grouped by (vertex, block)
   int* perm;      // [n_s * Ns]
   int* seg;       // [n_s * (maxnb + 1)]
+  int* count;     // [n_s * maxnb * chunks of 1024 samples] of the chunked sort; null: the other sort
   int* seg_v;     // [n_seg] vertex of segment
   int* seg_b;     // [n_seg] block of segment
   int maxnb, n_seg;
