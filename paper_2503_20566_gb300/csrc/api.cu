@@ -219,6 +219,7 @@ size_t group_smem_bytes(const Plan& p, int level, size_t sb) {
 }
 bool grouped(const gcf_ctx* c);
 int n_groups(const gcf_ctx* c);
+int chains_per_cta(const gcf_ctx* c, int n);
 
 void plan_group(gcf_ctx* c) {
   Plan& p = c->plan;
@@ -306,6 +307,17 @@ void append_derived_tables(const gcf_ctx* c, std::vector<int>& t) {
     t.push_back(r + 1 < R ? dense(&p.bondB[r * W], physB(r), &p.bondB[(r + 1) * W], physB(r + 1)) : 0);
   for (int r = 0; r < R; ++r)
     t.push_back(r + 1 < R ? dense(&p.bondT[(r + 1) * W], physT(r + 1), &p.bondT[r * W], physT(r)) : 0);
+}
+
+// Chains per CTA of the grouped forms for n chains: as many groups as it takes
+// to seat them all at once on the SMs, up to the form's.  A few chains then
+// have an SM each instead of sharing it four at a time (16 amplitudes on 3x3:
+// 140 -> 123 us; 256 chains of 6x6: 2.03 -> 1.79 ms); the arithmetic of a
+// chain does not depend on it.  The lockstep test hook needs its full CTA.
+int chains_per_cta(const gcf_ctx* c, int n) {
+  int W = n_groups(c);
+  while (W > 1 && (long long)n <= (long long)c->sms * (W / 2) && !c->lock_fault) W /= 2;
+  return W;
 }
 
 bool grouped(const gcf_ctx* c) { return c->exec == EXEC_GROUP || c->exec == EXEC_GROUP4; }
@@ -688,7 +700,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
                    int8_t* configs, const gcf_samples* out, int* gauss_count, cudaStream_t stream,
                    bool async) {
   const bool warp = grouped(c);
-  const int W = n_groups(c);  // chains per CTA
+  const int W = chains_per_cta(c, n);
   int grid = 1;
   if (warp) {
     const int per_sm = GCF_TC_CALL(T, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem);
@@ -708,6 +720,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
     k.tc_off = (long long)group_tc_off(c->plan, c->plan.group_level, c->sbytes);
     k.fz_off = (long long)group_fz_off(c->plan, c->plan.group_level, c->sbytes);
   }
+  if (warp && W == 1) k.lockstep = 0;
   k.n_chains = n; k.n_sweeps = n_sweeps; k.mode = mode; k.want = want; k.seed = seed;
   k.configs = configs;
   if (out) {
@@ -1387,7 +1400,7 @@ gcf_status gcf_sample_batch_async(gcf_ctx* c, int n_chains, int n_sweeps, uint64
   // scratch must already cover this launch: no allocation here
   {
     const bool grp = grouped(c);
-    const int W = n_groups(c);
+    const int W = chains_per_cta(c, n_chains);
     long long slots = 1;
     if (grp) {
       int per_sm = 0;
