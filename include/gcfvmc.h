@@ -83,7 +83,7 @@ enum { GCF_FP64 = 0, GCF_FP32 = 1, GCF_TF32 = 2, GCF_BF16 = 3 };
 /* parameter update of gcf_sr_step */
 enum { GCF_SR = 0, GCF_TDVP_STAGE1 = 1, GCF_TDVP_STAGE2 = 2 };
 /* truncation of the boundary MPS (gcf_model.trunc): the SVD sweep of
- * Sec. S-2 (QR left to right, then LQ / truncated SVD right to left).  A
+ * Sec. S-2 (QR left to right, then truncated SVD right to left).  A
  * randomized range finder is not built; any other value is GCF_EINVAL. */
 enum { GCF_TRUNC_SVD = 0 };
 
@@ -166,7 +166,7 @@ gcf_status gcf_init_configs(gcf_ctx* ctx, int n_chains, const int8_t* occupation
 
 /* Amplitude psi(s) = <B[Ly-2] | row Ly-1> where B[r] is the boundary MPS of
  * rows 0..r absorbed bottom-up, each compressed to chi by QR left-to-right
- * and LQ / truncated SVD right-to-left (Sec. S-2, Eq. S5; cost paragraph of
+ * and truncated SVD right-to-left (Sec. S-2, Eq. S5; cost paragraph of
  * the main text).  configs: device n*cfg_len; log_abs, phase: device [n].
  * An unphysical configuration gives log_abs = -inf, phase = 0 (its amplitude
  * is exactly zero in a GI-PEPS, Sec. S-2) and GCF_OK. */
@@ -309,7 +309,7 @@ int64_t gcf_launch_count(const gcf_ctx* ctx);
 
 /* Form of the sampling / measurement kernel this context launches (an
  * implementation choice; the paper has no counterpart): 0 = one chain per
- * CTA of 256 threads (gcf::vmc_kernel), 1 = two chains per CTA on groups of
+ * CTA of 256 or 512 threads (gcf::vmc_kernel), 1 = two chains per CTA on groups of
  * 128 threads (gcf::vmc_kernel_grouped), 2 = four chains per CTA of 512
  * threads (gcf::vmc_kernel_grouped4).  In the grouped forms the chain groups
  * of a CTA meet before every row of a pass (lockstep; bounded waits, no data

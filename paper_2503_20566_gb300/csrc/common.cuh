@@ -254,10 +254,9 @@ __shared__ int g_gemm_mode[4];
 //
 // TC: the executor of a kernel whose environment GEMMs may run on tcgen05 (the
 // BF16 form).  A kernel that holds tcgen05 instructions is given one block
-// per SM whatever its resources (the occupancy query's answer, and the
-// launches' behaviour: 118 -> 64 ms is what the second block is worth to 304
-// log-derivatives at 16x16, chi = 24), so the other forms' kernels are
-// compiled without them.
+// per SM whatever its resources (the occupancy query's answer), so the other
+// forms' kernels are compiled without them (304 log-derivatives at 16x16, chi =
+// 24, with the second block per SM: 64 -> 43 ms).
 template <bool TC = false>
 struct CtaExecT {
   static constexpr bool tc = TC;

@@ -11,8 +11,9 @@
 //
 // Measured against the same steps with every column in shared memory or L2 (a
 // barrier and a pass over the matrix per column or column pair) and Q and J
-// formed: log-derivatives at 16x16, chi = 24, 304 configurations 117.7 -> 73.4
-// ms; 10x10, D_k = 3, chi = 36, complex, 152 configurations 403 -> 161 ms.
+// formed: log-derivatives at 16x16, chi = 24, 304 configurations 117.7 -> 63.8
+// ms (43 with two blocks per SM); 10x10, D_k = 3, chi = 36, complex, 152
+// configurations 403 -> 159 ms (94 with 512 threads a chain).
 //
 // All matrices are column-major with leading dimensions padded to 4 rows
 // (pad4), so a lane moves 16 bytes of a column at a time.
@@ -584,7 +585,7 @@ __device__ __forceinline__ void apply_rot(T* a, T* b, typename Traits<T>::R c, T
 // blocks is held in the registers of LG lanes (R rows of each of the 8
 // columns a lane) while all 16 cross pairs (in the first round of a sweep also
 // the 12 pairs inside the blocks) are rotated, four disjoint pairs at a time.
-// Each quarter of the lanes forms the rotation of one pair; the squared norms
+// Each quarter of the lanes forms the rotation of one pair (quarter i that of a_i); the squared norms
 // are summed once per meeting and moved along by the rotations, so a step
 // reduces only the four inner products.  Returns the sweeps used.
 template <class T, int LG, int R, class X>
@@ -592,7 +593,7 @@ __device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int l
                                           int* converged) {
   using S = typename Traits<T>::R;
   const int nb = kp >> 2, npair = nb >> 1;
-  const int slots = ex.size() / LG, sub = ex.tid() / LG, li = ex.tid() & (LG - 1), quarter = li / (LG / 4);
+  const int slots = ex.size() / LG, sub = ex.tid() / LG, li = ex.tid() & (LG - 1);
   const S tol = S(4) * sqrt(S(p > 4 ? p : 4)) * Traits<T>::eps();
   // a column whose norm is below eps ||W||_F is rounding noise of the matrix:
   // pairs with one are left as they are
@@ -685,7 +686,6 @@ __device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int l
           }
           be = lane_of(be, (li + LG / 4) & (LG - 1), LG);
         }
-        (void)quarter;
         if (any) {
           rotated = true;
           if (act) {
