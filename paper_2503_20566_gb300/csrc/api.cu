@@ -801,9 +801,11 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     ks[i].fz_elems = fz;
     ks[i].fz_off = (long long)fz_off;
   }
-  // Four chains per CTA (vmc_kernel_multi4) when some context truncates: its
-  // sampling is bound by the latency of the factorisations, which more
-  // resident chains hide; hot buffers then stay in scratch (level 0).
+  // One chain per CTA (vmc_kernel_multi) where two CTAs fit an SM: 338 samples/s
+  // on the 16x16 + 24x24 + 32x32 boson mix (chi = 24) against 326 with four
+  // chains per CTA (vmc_kernel_multi4, hot buffers in scratch), and fewer
+  // chains spread over more SMs.  Truncating contexts whose shared memory or
+  // tcgen05 instructions leave one CTA per SM take four chains per CTA.
   // GCFVMC_MULTI=cta|group4 forces a form.
   int block = 256;
   long long group_bytes = 0;
@@ -813,7 +815,7 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     const size_t g_tc = (sharedv_bytes() + cfg_max + 15) / 16 * 16;
     const size_t g_fz = g_tc;
     const size_t gb = (g_tc + area + 15) / 16 * 16;
-    bool want4 = fz > 0;
+    bool want4 = fz > 0 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi, smem) < 2;
     if (const char* e = std::getenv("GCFVMC_MULTI")) want4 = !std::strcmp(e, "group4");
     if (want4 && 4 * gb <= 216 * 1024 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi4, 4 * gb) >= 1) {
       block = 512;
