@@ -309,15 +309,24 @@ int64_t gcf_launch_count(const gcf_ctx* ctx);
 
 /* Form of the sampling / measurement kernel this context launches (an
  * implementation choice; the paper has no counterpart): 0 = one chain per
- * CTA of 256 or 512 threads (gcf::vmc_kernel), 1 = two chains per CTA on groups of
- * 128 threads (gcf::vmc_kernel_grouped), 2 = four chains per CTA of 512
- * threads (gcf::vmc_kernel_grouped4).  In the grouped forms the chain groups
- * of a CTA meet before every row of a pass (lockstep; bounded waits, no data
- * exchanged), so the SM runs one region of code at a time.  Chosen at
- * context creation from the shared-memory footprint (or by gcf_autotune);
- * GCFVMC_EXEC=cta|group|group4 and GCFVMC_LOCK=0|1 in the environment force
- * a form.  All forms compute the same results. */
+ * CTA of 256 or 512 threads (gcf::vmc_kernel), 1 = up to two chains per CTA on
+ * groups of 128 threads (gcf::vmc_kernel_grouped), 2 = up to four chains per
+ * CTA (gcf::vmc_kernel_grouped4; gcf::vmc_kernel_grouped for one or two).  The
+ * grouped forms take the fewest chains per CTA that seat all chains of the
+ * call on the SMs at once (n <= SMs: one; n <= 2 SMs: two).  With several, the
+ * chain groups of a CTA meet before every row of a pass (lockstep; bounded
+ * waits, no data exchanged), so the SM runs one region of code at a time.
+ * Chosen at context creation from the shared-memory footprint (or by
+ * gcf_autotune); GCFVMC_EXEC=cta|group|group4 and GCFVMC_LOCK=0|1 in the
+ * environment force a form, with its full chains per CTA for any n.  All forms
+ * compute the same results. */
 int gcf_executor(const gcf_ctx* ctx);
+
+/* Chains per CTA of this context's last launch of that kernel (implementation
+ * detail, no counterpart in the paper): 1, 2 or 4; 0 before any launch with
+ * the present form, -1 for a NULL context.  (gcf_sample_multi has
+ * gcf_multi_chains_per_cta.) */
+int gcf_chains_per_cta(const gcf_ctx* ctx);
 
 /* Lockstep waits that ran out in the last synchronous sampling or
  * measurement launch of this context (implementation detail; no counterpart

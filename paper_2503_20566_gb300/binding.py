@@ -64,6 +64,7 @@ def load_library(path: str = LIB_PATH):
         "gcf_scalar_bytes": (i, [vp]),
         "gcf_launch_count": (i64, [vp]),
         "gcf_executor": (i, [vp]),
+        "gcf_chains_per_cta": (i, [vp]),
         "gcf_smem_level": (i, [vp]),
         "gcf_phase_timeouts": (i, [vp]),
         "gcf_svd_unconverged": (i, [vp]),
@@ -99,7 +100,7 @@ def load_library(path: str = LIB_PATH):
 def exported_symbols():
     """Names the binding expects the library to export."""
     return ["gcf_init_peps", "gcf_destroy", "gcf_last_error", "gcf_num_params", "gcf_config_len",
-            "gcf_scalar_bytes", "gcf_launch_count", "gcf_executor", "gcf_smem_level", "gcf_phase_timeouts", "gcf_svd_unconverged", "gcf_set_svd_sweeps", "gcf_scratch_bytes_per_chain", "gcf_checkpoint_interval", "gcf_tensor_core_form", "gcf_tensor_timeouts", "gcf_multi_chains_per_cta", "gcf_autotune", "gcf_set_tensors", "gcf_get_tensors",
+            "gcf_scalar_bytes", "gcf_launch_count", "gcf_executor", "gcf_chains_per_cta", "gcf_smem_level", "gcf_phase_timeouts", "gcf_svd_unconverged", "gcf_set_svd_sweeps", "gcf_scratch_bytes_per_chain", "gcf_checkpoint_interval", "gcf_tensor_core_form", "gcf_tensor_timeouts", "gcf_multi_chains_per_cta", "gcf_autotune", "gcf_set_tensors", "gcf_get_tensors",
             "gcf_init_configs", "gcf_amplitude", "gcf_local_energy", "gcf_log_grad", "gcf_log_grad_vjp", "gcf_sample_multi",
             "gcf_sample_batch", "gcf_sample_batch_async", "gcf_sr_step", "gcf_vmc_step_host"]
 
@@ -276,10 +277,18 @@ class Context:
         return int(self.lib.gcf_smem_level(self.ctx))
 
     @property
+    def chains_per_cta(self):
+        """Chains per CTA of the last sampling / measurement launch (0 before any)."""
+        return int(self.lib.gcf_chains_per_cta(self.ctx))
+
+    @property
     def kernel_name(self):
-        """Name of the sampling / measurement kernel this context launches."""
-        return {1: "gcf::vmc_kernel_grouped", 2: "gcf::vmc_kernel_grouped4"}.get(
-            int(self.lib.gcf_executor(self.ctx)), "gcf::vmc_kernel")
+        """Name of the sampling / measurement kernel of the last launch; before
+        any, of the one that many chains take."""
+        if int(self.lib.gcf_executor(self.ctx)) == 0:
+            return "gcf::vmc_kernel"
+        few = self.chains_per_cta in (1, 2) or int(self.lib.gcf_executor(self.ctx)) == 1
+        return "gcf::vmc_kernel_grouped" if few else "gcf::vmc_kernel_grouped4"
 
     # ---- parameters -------------------------------------------------------
     def set_tensors(self, values):

@@ -72,10 +72,12 @@ struct gcf_ctx {
   int lockstep = 0;  // grouped kernels: chain groups of a CTA in lockstep
   int ck_every = 0;  // boundary-MPS store: keep every K-th slot and recompute between (0: keep all)
   int lock_fault = 0;  // test hook (GCFVMC_LOCK_FAULT): one group never counts in
+  int forced = 0;      // GCFVMC_EXEC chose the form: keep its chains per CTA whatever their number
   int last_phase_timeouts = 0;
   int last_svd_unconverged = 0;  // SVDs that hit the sweep limit in the last synchronous launch
   int last_tc_timeouts = 0;      // tensor-core waits that ran out in the last synchronous launch
   int last_multi_block = 0;      // block size of the last gcf_sample_multi launch (256 or 512)
+  int last_chains = 0;           // chains per CTA of the last launch of vmc_kernel / _grouped / _grouped4 (0: none)
   int svd_sweeps = 40;           // sweep limit of the one-sided Jacobi SVD
   int tab_ints = 0;  // ints in d_tables
   // device
@@ -260,6 +262,7 @@ void plan_group(gcf_ctx* c) {
       p.group_level = lv2;
     }
     if (!std::strcmp(e, "cta")) c->exec = EXEC_CTA;
+    c->forced = 1;
   }
   if (const char* e = std::getenv("GCFVMC_SMEM")) p.group_level = std::max(0, std::min(3, std::atoi(e)));
   p.group_smem = group_smem_bytes(p, p.group_level, c->sbytes);
@@ -313,10 +316,11 @@ void append_derived_tables(const gcf_ctx* c, std::vector<int>& t) {
 // to seat them all at once on the SMs, up to the form's.  A few chains then
 // have an SM each instead of sharing it four at a time (16 amplitudes on 3x3:
 // 140 -> 123 us; 256 chains of 6x6: 2.03 -> 1.79 ms); the arithmetic of a
-// chain does not depend on it.  The lockstep test hook needs its full CTA.
+// chain does not depend on it.  A form that GCFVMC_EXEC forced keeps its groups,
+// and so does the lockstep test hook.
 int chains_per_cta(const gcf_ctx* c, int n) {
   int W = n_groups(c);
-  while (W > 1 && (long long)n <= (long long)c->sms * (W / 2) && !c->lock_fault) W /= 2;
+  while (W > 1 && (long long)n <= (long long)c->sms * (W / 2) && !c->forced && !c->lock_fault) W /= 2;
   return W;
 }
 
@@ -327,6 +331,7 @@ int n_groups(const gcf_ctx* c) { return c->exec == EXEC_GROUP4 ? 4 : 2; }
 void set_form(gcf_ctx* c, int exec, int level) {
   Plan& p = c->plan;
   c->exec = exec;
+  c->last_chains = 0;
   if (exec == EXEC_GROUP || exec == EXEC_GROUP4) {
     p.group_level = level;
     p.group_smem = group_smem_bytes(p, level, c->sbytes);
@@ -734,6 +739,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
   else
     CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc, k, grid, cta_block(c, n), c->plan.dyn_smem, stream));
   c->launches += 1;
+  c->last_chains = warp ? W : 1;
   if (async) return GCF_OK;
   int h_status[4];
   CUDA_TRY(c, cudaMemcpyAsync(h_status, c->d_status, sizeof(h_status), cudaMemcpyDeviceToHost, c->stream));
@@ -1132,6 +1138,8 @@ int gcf_scalar_bytes(const gcf_ctx* c) { return c ? (int)c->sbytes : -1; }
 int64_t gcf_launch_count(const gcf_ctx* c) { return c ? c->launches : -1; }
 
 int gcf_executor(const gcf_ctx* ctx) { return ctx ? ctx->exec : -1; }
+
+int gcf_chains_per_cta(const gcf_ctx* ctx) { return ctx ? ctx->last_chains : -1; }
 
 gcf_status gcf_set_tensors(gcf_ctx* c, const void* host, size_t bytes) {
   if (!c || !host) return GCF_EINVAL;

@@ -1,0 +1,49 @@
+"""The kernel form that runs is the one asked for, and the one reported.
+
+A grouped form seats the chains of a call on as few chains per CTA as the SMs
+allow; a form forced by GCFVMC_EXEC keeps its own number, so that the tests
+which force one run it.  chains_per_cta and kernel_name report the launch.
+"""
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_helpers import oracle_net
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("form,per_cta,name", [("cta", 1, "gcf::vmc_kernel"), ("group", 2, "gcf::vmc_kernel_grouped"),
+                                               ("group4", 4, "gcf::vmc_kernel_grouped4")])
+def test_forced_form_keeps_its_chains_per_cta(form, per_cta, name, monkeypatch):
+    import paper_2503_20566_gb300 as G
+
+    monkeypatch.setenv("GCFVMC_EXEC", form)
+    ctx = G.Context(2, 4, 4, 4, 4, g=0.4, seed=1)
+    for n in (1, 3, 5):
+        ctx.amplitude(ctx.init_configs(n))
+        assert (ctx.chains_per_cta, ctx.kernel_name) == (per_cta, name), n
+
+
+def test_default_form_spreads_few_chains_and_leaves_them_unchanged():
+    import paper_2503_20566_gb300 as G
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lat, _, vals = oracle_net(4, 4, 2, 4, seed=41)
+    n = 4 * sms + 1
+    ctx = G.Context(2, 4, 4, 4, 4, g=0.4, seed=1)
+    ctx.set_tensors(vals)
+    start = ctx.init_configs(n, None, synth.plaquette_powers(42, n, lat.n_plaquettes, 2))
+    ref = None
+    for m, per_cta in ((n, 4), (2 * sms + 1, 4), (2 * sms, 2), (sms + 1, 2), (sms, 1), (5, 1), (1, 1)):
+        cfg = start[:m].clone()
+        out = ctx.sample_batch(cfg, 1, 7)
+        assert ctx.chains_per_cta == per_cta, m
+        assert ctx.kernel_name == "gcf::vmc_kernel_grouped" + ("4" if per_cta == 4 else ""), m
+        got = [cfg] + [out[k].reshape(m, -1) for k in ("log_abs", "e_loc", "O", "accepted")]
+        ref = ref or got
+        for a, b in zip(got, ref):
+            assert np.array_equal(a.cpu().numpy(), b[:m].cpu().numpy()), m
