@@ -391,7 +391,9 @@ int gcf_smem_level(const gcf_ctx* ctx);
  * kernel form that fits an SM (executor x shared-memory level) on
  * gcf_sample_batch of a copy of `configs` (device, n_chains x cfg_len, left
  * unchanged) for n_sweeps sweeps, after one warm-up run per form, and keeps
- * the fastest for this context's later launches.  ms (host, optional): the
+ * the fastest for this context's later launches.  Up to two chains per SM the
+ * two grouped forms of a level are the same launch: it is timed once, as form
+ * 1 of gcf_executor.  ms (host, optional): the
  * time of form i (1e300 if it did not launch) for i < *n_forms on entry;
  * *n_forms (optional) is set to the number of forms tried.  Allocates and
  * frees its own work buffers; synchronises the context's stream. */

@@ -679,6 +679,16 @@ int grid_for(gcf_ctx* c, int n_chains) {
   return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm));
 }
 
+// Resident CTAs per SM of the grouped kernel with W chain groups.
+int grouped_per_sm(const gcf_ctx* c, int W, size_t smem) {
+  switch (c->kind) {
+    case S_F32: return GCF_TC_CALL(float, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
+    case S_F64: return GCF_TC_CALL(double, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
+    case S_C64: return GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
+    default: return GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
+  }
+}
+
 // cudaMalloc that leaves the pointer null when it fails (retry paths free
 // whatever a group holds)
 template <class P>
@@ -1284,17 +1294,29 @@ gcf_status gcf_log_grad_vjp(gcf_ctx* c, int n, const int8_t* configs, const doub
 gcf_status gcf_autotune(gcf_ctx* c, int n_chains, int n_sweeps, const int8_t* configs, double* ms, int* n_forms) {
   if (!c || n_chains < 1 || n_sweeps < 1 || !configs) return GCF_EINVAL;
   DEVICE_TRY(c, "gcf_autotune");
-  // candidate forms that fit an SM (227 KB of shared memory per block)
+  // candidate forms that fit an SM (227 KB of shared memory per block), a
+  // grouped one with all its groups: the timing may run fewer (chains_per_cta),
+  // later calls with more chains do not
   const size_t limit = 227 * 1024 - 8 * 1024;
+  const int keep_exec = c->exec, keep_cta = c->plan.cta_level, keep_grp = c->plan.group_level;
   std::vector<std::pair<int, int>> forms;
   for (int lv = 0; lv <= 3; ++lv) {
     const size_t cta = cta_smem_bytes(c->plan, lv, c->sbytes);
     if (cta <= limit) forms.push_back({EXEC_CTA, lv});
     const size_t grp = 2 * group_smem_bytes(c->plan, lv, c->sbytes);
-    if (lv >= 1 && grp <= limit) forms.push_back({EXEC_GROUP, lv});
-    if (lv >= 1 && 2 * grp <= limit) forms.push_back({EXEC_GROUP4, lv});
+    int two = 0;  // chains per CTA that two groups take for n_chains
+    for (int ex : {EXEC_GROUP, EXEC_GROUP4}) {
+      const size_t smem = ex == EXEC_GROUP ? grp : 2 * grp;
+      if (lv < 1 || smem > limit) continue;
+      c->exec = ex;
+      const int seat = chains_per_cta(c, n_chains);
+      // so few chains that both grouped forms are the same launch: timed once
+      if (ex == EXEC_GROUP4 && seat == two) continue;
+      if (ex == EXEC_GROUP) two = seat;
+      if (grouped_per_sm(c, n_groups(c), smem) >= 1) forms.push_back({ex, lv});
+    }
   }
-  const int keep_exec = c->exec, keep_cta = c->plan.cta_level, keep_grp = c->plan.group_level;
+  c->exec = keep_exec;
   const size_t bytes = (size_t)n_chains * c->cfg_len;
   int8_t* work = nullptr;
   double* la = nullptr;
@@ -1413,13 +1435,7 @@ gcf_status gcf_sample_batch_async(gcf_ctx* c, int n_chains, int n_sweeps, uint64
     const int W = chains_per_cta(c, n_chains);
     long long slots = 1;
     if (grp) {
-      int per_sm = 0;
-      switch (c->kind) {
-        case S_F32: per_sm = GCF_TC_CALL(float, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
-        case S_F64: per_sm = GCF_TC_CALL(double, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
-        case S_C64: per_sm = GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
-        default: per_sm = GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem); break;
-      }
+      const int per_sm = grouped_per_sm(c, W, W * c->plan.group_smem);
       const long long sl = balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm) * W);
       slots = (sl + W - 1) / W * W;
     } else {

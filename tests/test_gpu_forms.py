@@ -2,7 +2,8 @@
 
 A grouped form seats the chains of a call on as few chains per CTA as the SMs
 allow; a form forced by GCFVMC_EXEC keeps its own number, so that the tests
-which force one run it.  chains_per_cta and kernel_name report the launch.
+which force one run it.  chains_per_cta and kernel_name report the launch, and the
+autotuner times no launch under two names.
 """
 
 import numpy as np
@@ -47,3 +48,16 @@ def test_default_form_spreads_few_chains_and_leaves_them_unchanged():
         ref = ref or got
         for a, b in zip(got, ref):
             assert np.array_equal(a.cpu().numpy(), b[:m].cpu().numpy()), m
+
+
+@pytest.mark.parametrize("per_sm,forms", [(1, 4 + 3), (2, 4 + 3), (3, 4 + 3 + 3)])
+def test_autotune_times_each_launch_once(per_sm, forms):
+    """One-chain-per-CTA at four levels, two groups at three; four groups only
+    where the chains outnumber two per SM (below, the launches would be the
+    same and noise would choose the name)."""
+    import paper_2503_20566_gb300 as G
+
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    ctx = G.Context(2, 3, 3, 4, 4, g=0.4, seed=1)
+    assert len(ctx.autotune(ctx.init_configs(n))) == forms
+    assert per_sm > 2 or ctx.kernel_name != "gcf::vmc_kernel_grouped4"
