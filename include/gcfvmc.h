@@ -260,7 +260,9 @@ gcf_status gcf_sample_batch_async(gcf_ctx* ctx, int n_chains, int n_sweeps, uint
  * (n_chains > 1, else over samples), CG iterations, relative residual,
  * |F|, 1 if CG reached tol, 1 if the diagonal preconditioner was used};
  * n_chains is the number of chains the samples came from
- * (chain-major order).  GCF_ETIMEOUT if CG hits max_iter before tol (the
+ * (chain-major order).  GCF_EINVAL, with the tensors unchanged, if some
+ * block id names no block of its vertex (block_ids of a chain that did not
+ * run, say).  GCF_ETIMEOUT if CG hits max_iter before tol (the
  * update is still applied).  Sums over samples and dot products combine
  * per-block partial sums with FP64 atomics, so repeated calls on the same
  * samples agree to rounding, not bit for bit. */

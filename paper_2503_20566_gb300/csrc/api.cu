@@ -1021,7 +1021,7 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
         !dalloc(&c->sr.osort, c->sbytes * (size_t)Ns * c->sr_sum_bs))
       return fail(c, GCF_ENOMEM, "SR sample vectors");
     // the chunked sort's table, where it is small beside the rest (else the sort that needs none)
-    if (c->sr.maxnb <= 128 && !dalloc(&c->sr.count, sizeof(int) * (size_t)c->n_s * c->sr.maxnb * ((Ns + 1023) / 1024)))
+    if (c->sr.maxnb <= 128 && !dalloc(&c->sr.count, sizeof(int) * (size_t)c->n_s * (c->sr.maxnb + 1) * ((Ns + 1023) / 1024)))
       return fail(c, GCF_ENOMEM, "SR sample vectors");
     c->sr_ns_cap = Ns;
   }
@@ -1496,24 +1496,26 @@ gcf_status gcf_sr_step(gcf_ctx* c, int n_samples, int n_chains, const double* e_
   for (int v = 0; v < c->n_s; ++v) mx = std::max(mx, c->vbs[v] * c->vnb[v]);
   g.max_nb_bs = mx;
   cudaError_t e;
+  bool bad_ids = false;
   switch (c->kind) {
     case S_F32:
       e = sr_solve_update<float>(g, c->sr, e_loc, block_ids, O, c->d_params, n_chains, diag_shift, cr, ci,
-                                 max_iter, tol, stats, c->stream, &c->launches);
+                                 max_iter, tol, stats, &bad_ids, c->stream, &c->launches);
       break;
     case S_F64:
       e = sr_solve_update<double>(g, c->sr, e_loc, block_ids, O, c->d_params, n_chains, diag_shift, cr, ci,
-                                  max_iter, tol, stats, c->stream, &c->launches);
+                                  max_iter, tol, stats, &bad_ids, c->stream, &c->launches);
       break;
     case S_C64:
       e = sr_solve_update<cfloat>(g, c->sr, e_loc, block_ids, O, c->d_params, n_chains, diag_shift, cr, ci,
-                                  max_iter, tol, stats, c->stream, &c->launches);
+                                  max_iter, tol, stats, &bad_ids, c->stream, &c->launches);
       break;
     default:
       e = sr_solve_update<cdouble>(g, c->sr, e_loc, block_ids, O, c->d_params, n_chains, diag_shift, cr, ci,
-                                   max_iter, tol, stats, c->stream, &c->launches);
+                                   max_iter, tol, stats, &bad_ids, c->stream, &c->launches);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "gcf_sr_step");
+  if (bad_ids) return fail(c, GCF_EINVAL, "gcf_sr_step: block_ids names a block that its vertex does not have");
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   if (stats[6] == 0.0 && max_iter > 0) return fail(c, GCF_ETIMEOUT, "CG reached max_iter before tol");
   return GCF_OK;

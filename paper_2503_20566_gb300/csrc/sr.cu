@@ -97,6 +97,7 @@ __global__ void k_mean_err(const cdouble* v, int m, double* out) {
     out[0] = mr;
     out[1] = mi;
     out[2] = m > 1 ? sqrt(q / (m - 1) / m) : 0.0;
+    out[3] = 0.0;  // set by the sort if it meets a block id that the vertex does not have
   }
 }
 
@@ -227,9 +228,11 @@ __global__ void k_update(T* params, const cdouble* x, double cr, double ci, long
 // Sample order grouped by (vertex, block): for every vertex a stable counting
 // sort of the samples by the block they select.  seg[v * (maxnb + 1) + b] is
 // the start of block b of vertex v inside perm[v * Ns ...]; built once per SR
-// step (block ids do not change during the solve).  One CTA per vertex.
+// step (block ids do not change during the solve).  Samples whose id names no
+// block of the vertex come last, behind seg[.. + nb], and set *bad: the step
+// stops before anything is read through such an id.  One CTA per vertex.
 // ---------------------------------------------------------------------------
-__global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm, int* seg) {
+__global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm, int* seg, double* bad) {
   __shared__ int wsum[32];
   __shared__ int base_s;
   const int v = blockIdx.x;
@@ -239,12 +242,16 @@ __global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm,
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (threadIdx.x == 0) base_s = 0;
   __syncthreads();
-  for (int b = 0; b < nb; ++b) {
-    if (threadIdx.x == 0) seg[v * (maxnb + 1) + b] = base_s;
+  for (int b = 0; b <= nb; ++b) {
+    if (threadIdx.x == 0) {
+      seg[v * (maxnb + 1) + b] = base_s;
+      if (b == nb && base_s < Ns) *bad = 1.0;
+    }
     __syncthreads();
     for (long long s0 = 0; s0 < Ns; s0 += blockDim.x) {
       const long long s = s0 + threadIdx.x;
-      const int hit = (s < Ns && bids[s * g.n_s + v] == b) ? 1 : 0;
+      const int id = s < Ns ? bids[s * g.n_s + v] : -1;
+      const int hit = (s < Ns && (b < nb ? id == b : (unsigned)id >= (unsigned)nb)) ? 1 : 0;
       // block-wide exclusive scan of hit (stable order)
       const unsigned m = __ballot_sync(0xffffffffu, hit);
       const int before = __popc(m & ((1u << lane) - 1u));
@@ -261,19 +268,21 @@ __global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm,
       __syncthreads();
     }
   }
-  if (threadIdx.x == 0) seg[v * (maxnb + 1) + nb] = base_s;
 }
 
 // The same order from three passes over chunks of 1024 samples, for at most
 // kSortBlocks blocks a vertex (one CTA per vertex walks all samples once per
-// block above: 905 us at 65536 samples on 8x8, this 40).  count: [vertex][block]
-// [chunk], turned from counts into starts by the middle pass.
+// block above: 905 us at 65536 samples on 8x8, this 40).  count: [vertex][block,
+// and one row for ids that are no block][chunk], turned from counts into starts
+// by the middle pass.
 constexpr int kSortBlocks = 128;
+// nb: the vertex's blocks and the row of the others
 __device__ __forceinline__ int sort_rank(const int* bids, const SrGeom& g, int v, int nb, int* wcnt, int& b, bool& in) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long s = (long long)blockIdx.x * 1024 + threadIdx.x;
   in = s < g.Ns;
   b = in ? bids[s * g.n_s + v] : -1;
+  if (in && (unsigned)b >= (unsigned)(nb - 1)) b = nb - 1;
   for (int i = threadIdx.x; i < 32 * nb; i += 1024) wcnt[i] = 0;
   __syncthreads();
   const unsigned m = __match_any_sync(0xffffffffu, b);
@@ -284,20 +293,20 @@ __device__ __forceinline__ int sort_rank(const int* bids, const SrGeom& g, int v
 }
 __global__ void k_sort_count(SrGeom g, const int* bids, int maxnb, int n_chunk, int* count) {
   extern __shared__ int wcnt[];
-  const int v = blockIdx.y, nb = g.vnb[v];
+  const int v = blockIdx.y, nb = g.vnb[v] + 1;
   int b;
   bool in;
   sort_rank(bids, g, v, nb, wcnt, b, in);
   for (int i = threadIdx.x; i < nb; i += 1024) {
     int t = 0;
     for (int w = 0; w < 32; ++w) t += wcnt[w * nb + i];
-    count[((long long)v * maxnb + i) * n_chunk + blockIdx.x] = t;
+    count[((long long)v * (maxnb + 1) + i) * n_chunk + blockIdx.x] = t;
   }
 }
-__global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* seg) {
+__global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* seg, double* bad) {
   __shared__ int tot[kSortBlocks + 1];
-  const int v = blockIdx.x, nb = g.vnb[v], lane = threadIdx.x & 31;
-  int* cv = count + (long long)v * maxnb * n_chunk;
+  const int v = blockIdx.x, nb = g.vnb[v] + 1, lane = threadIdx.x & 31;
+  int* cv = count + (long long)v * (maxnb + 1) * n_chunk;
   for (int b = threadIdx.x >> 5; b < nb; b += blockDim.x >> 5) {
     int t = 0;
     for (int i = lane; i < n_chunk; i += 32) t += cv[b * n_chunk + i];
@@ -312,8 +321,8 @@ __global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* s
       tot[b] = acc;
       seg[v * (maxnb + 1) + b] = acc;
       acc += t;
+      if (b == nb - 1 && t > 0) *bad = 1.0;
     }
-    seg[v * (maxnb + 1) + nb] = acc;
   }
   __syncthreads();
   for (int b = threadIdx.x >> 5; b < nb; b += blockDim.x >> 5) {
@@ -332,12 +341,12 @@ __global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* s
 }
 __global__ void k_sort_place(SrGeom g, const int* bids, int maxnb, int n_chunk, const int* count, int* perm) {
   extern __shared__ int wcnt[];
-  const int v = blockIdx.y, nb = g.vnb[v];
+  const int v = blockIdx.y, nb = g.vnb[v] + 1;
   int b;
   bool in;
   const int before = sort_rank(bids, g, v, nb, wcnt, b, in);
   for (int i = threadIdx.x; i < nb; i += 1024) {
-    int t = count[((long long)v * maxnb + i) * n_chunk + blockIdx.x];
+    int t = count[((long long)v * (maxnb + 1) + i) * n_chunk + blockIdx.x];
     for (int w = 0; w < 32; ++w) {
       const int c = wcnt[w * nb + i];
       wcnt[w * nb + i] = t;
@@ -798,7 +807,7 @@ static cudaError_t dot(const cdouble* a, const cdouble* b, long long n, double* 
 template <class T>
 cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, const int* bids,
                             const void* Ov, void* params, int n_chains, double shift, double cr,
-                            double ci, int max_iter, double tol, double* stats, cudaStream_t st,
+                            double ci, int max_iter, double tol, double* stats, bool* bad_ids, cudaStream_t st,
                             long long* launches) {
   const T* O = (const T*)Ov;
   const long long Np = g.Np, Ns = g.Ns;
@@ -832,13 +841,13 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   if (w.count) {
     const int n_chunk = nblk(Ns, 1024);
     const dim3 grid((unsigned)n_chunk, (unsigned)g.n_s);
-    const size_t smem = sizeof(int) * 32 * w.maxnb;
+    const size_t smem = sizeof(int) * 32 * (w.maxnb + 1);
     k_sort_count<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count);
-    k_sort_scan<<<g.n_s, 256, 0, st>>>(g, w.maxnb, n_chunk, w.count, w.seg);
+    k_sort_scan<<<g.n_s, 256, 0, st>>>(g, w.maxnb, n_chunk, w.count, w.seg, w.scal + 3);
     k_sort_place<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count, w.perm);
     *launches += 3;
   } else {
-    k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg);
+    k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg, w.scal + 3);
     ++*launches;
   }
   // O in segment order, streamed by every scatter of this step
@@ -891,6 +900,8 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   double h_sc[16];
   CK(cudaMemcpyAsync(h_sc, w.scal, 16 * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  *bad_ids = h_sc[3] != 0.0;
+  if (*bad_ids) return cudaSuccess;
   const double e_re = h_sc[0], e_im = h_sc[1], e_err = h_sc[2];
   const double rr0 = h_sc[8 + 6];
   const double fnorm = sqrt(rr0);
@@ -1001,15 +1012,15 @@ template cudaError_t log_grad_vjp<cdouble>(const SrGeom&, const int*, const void
 
 template cudaError_t sr_solve_update<float>(const SrGeom&, SrWork&, const double*, const int*,
                                             const void*, void*, int, double, double, double, int,
-                                            double, double*, cudaStream_t, long long*);
+                                            double, double*, bool*, cudaStream_t, long long*);
 template cudaError_t sr_solve_update<double>(const SrGeom&, SrWork&, const double*, const int*,
                                              const void*, void*, int, double, double, double, int,
-                                             double, double*, cudaStream_t, long long*);
+                                             double, double*, bool*, cudaStream_t, long long*);
 template cudaError_t sr_solve_update<cfloat>(const SrGeom&, SrWork&, const double*, const int*,
                                              const void*, void*, int, double, double, double, int,
-                                             double, double*, cudaStream_t, long long*);
+                                             double, double*, bool*, cudaStream_t, long long*);
 template cudaError_t sr_solve_update<cdouble>(const SrGeom&, SrWork&, const double*, const int*,
                                               const void*, void*, int, double, double, double, int,
-                                              double, double*, cudaStream_t, long long*);
+                                              double, double*, bool*, cudaStream_t, long long*);
 
 }  // namespace gcf

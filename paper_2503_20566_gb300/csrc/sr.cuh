@@ -31,7 +31,7 @@ struct SrWork {
   // sample order grouped by (vertex, block)
   int* perm;      // [n_s * Ns]
   int* seg;       // [n_s * (maxnb + 1)]
-  int* count;     // [n_s * maxnb * chunks of 1024 samples] of the chunked sort; null: the other sort
+  int* count;     // [n_s * (maxnb + 1) * chunks of 1024 samples] of the chunked sort; null: the other sort
   int* seg_v;     // [n_seg] vertex of segment
   int* seg_b;     // [n_seg] block of segment
   int maxnb, n_seg;
@@ -47,11 +47,12 @@ struct SrWork {
 };
 
 // Computes <E>, F, solves (S + shift) x = F by CG, then params += (cr + i ci) x.
-// stats[8] as documented for gcf_sr_step.
+// stats[8] as documented for gcf_sr_step.  *bad_ids: some block id names no block
+// of its vertex; nothing is updated then.
 template <class T>
 cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, const int* bids,
                             const void* O, void* params, int n_chains, double shift, double cr,
-                            double ci, int max_iter, double tol, double* stats, cudaStream_t st,
+                            double ci, int max_iter, double tol, double* stats, bool* bad_ids, cudaStream_t st,
                             long long* launches);
 
 // grad = sum_s w_s O_s scattered into the parameter layout (real: grad[Np],
