@@ -49,6 +49,7 @@ struct Plan {
   long long tc_bytes = 0;
   // shared-memory factorisation workspace of one chain (scalars; 0: none)
   long long fz_elems = 0;
+  bool general = false;  // some factorisation is beyond the register forms
   long long level_elems(int lv) const {
     return lv <= 0 ? 0 : lv == 1 ? hot_base_elems : lv == 2 ? hot_mps_elems : hot_all_elems;
   }
@@ -379,6 +380,11 @@ void build_plan(gcf_ctx* c) {
   auto vb = [&](long long m) { return 2 * ((m + rc - 1) / rc * rc) + 4; };
   auto p4 = [](long long n) { return (n + 3) & ~3LL; };
   bool truncates = false;
+  p.general = false;
+  const int max_qr = c->kind == S_F32 ? qr_max_rows<float>() : c->kind == S_F64 ? qr_max_rows<double>()
+                     : c->kind == S_C64 ? qr_max_rows<cfloat>() : qr_max_rows<cdouble>();
+  const int max_jac = c->kind == S_F32 ? jacobi_max_rows<float>() : c->kind == S_F64 ? jacobi_max_rows<double>()
+                      : c->kind == S_C64 ? jacobi_max_rows<cfloat>() : jacobi_max_rows<cdouble>();
   auto step_sizes = [&](const int* bin, const int* qr, const int* svd, const int* bout, int pout) {
     long long A = 1, q = 0;
     for (int cc = 1; cc < Lx; ++cc) A = std::max(A, (long long)bin[cc] * Dk);
@@ -389,6 +395,7 @@ void build_plan(gcf_ctx* c) {
       if (rows > cols) {
         q += (p4(rows) + 1) * cols + 32;
         fz_vb = std::max(fz_vb, vb(rows));
+        p.general |= rows > max_qr;
       }
       q = (q + 31) & ~31LL;
     }
@@ -396,6 +403,7 @@ void build_plan(gcf_ctx* c) {
     for (int cc = Lx - 1; cc >= 1; --cc) {
       if (!svd[cc]) continue;
       truncates = true;
+      p.general |= qr[cc] > max_qr || (long long)pout * bout[cc + 1] > max_jac;
       const long long yr = qr[cc], yc = (long long)pout * bout[cc + 1], k0 = std::min(yr, yc), kk = bout[cc];
       const long long w = vb(yr) + p4(yc) * ((k0 + 7) & ~7LL);
       fz_w = std::max(fz_w, w);
@@ -663,9 +671,13 @@ bool uses_tc(const gcf_ctx* c) { return c->plan.tc_bytes > 0; }
 
 // Threads per CTA of vmc_kernel for n chains: with at most one chain per SM a
 // truncating plan takes 512, since its factorisations and products have work
-// for more than 256 (the results are the same either way; plans that do not
-// truncate lose more in the barriers than they gain).
-int cta_block(const gcf_ctx* c, int n_chains) { return c->plan.fz_elems > 0 && n_chains <= c->sms ? 512 : 256; }
+// for more than 256 (plans that do not truncate lose more in the barriers than
+// they gain).  The register factorisations give the same results either way;
+// the general ones do not, and gain nothing (amplitudes 8x4, D_k = 3, chi = 22,
+// complex FP64: 17.4 ms with 512, 11.1 with 256), so their plans keep 256.
+int cta_block(const gcf_ctx* c, int n_chains) {
+  return c->plan.fz_elems > 0 && !c->plan.general && n_chains <= c->sms ? 512 : 256;
+}
 
 int grid_for(gcf_ctx* c, int n_chains) {
   int per_sm = 1;

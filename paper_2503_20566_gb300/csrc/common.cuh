@@ -263,7 +263,8 @@ struct CtaExecT {
   __device__ int tid() const { return threadIdx.x; }
   __device__ int size() const { return blockDim.x; }
   // threads among which the terms of a sum are dealt out: the same for every
-  // block size from 256, so that the results do not depend on it
+  // block size from 256, so that the results do not depend on it (the general
+  // QR and Jacobi of linalg.cuh deal to all threads; their plans have one size)
   __device__ int sum_size() const { return min((int)blockDim.x, 256); }
   __device__ int lane() const { return threadIdx.x & 31; }
   __device__ int warp() const { return threadIdx.x >> 5; }

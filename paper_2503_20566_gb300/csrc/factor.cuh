@@ -421,6 +421,15 @@ __host__ __device__ inline int qr_vb_elems(int m) {
   return 2 * ((m + RC - 1) / RC * RC) + 4;
 }
 
+// Longest columns that the register forms of the QR and of the Jacobi take.  The
+// general forms behind them deal their sums to all threads of the executor, so
+// their last bits depend on its size: a plan that reaches one keeps one block
+// size (see cta_block).
+template <class T>
+constexpr int qr_max_rows() { return Chunk<T>::ROWS * (sizeof(T) == 4 ? 11 : sizeof(T) == 8 ? 21 : 16); }
+template <class T>
+constexpr int jacobi_max_rows() { return sizeof(T) == 4 ? 256 : sizeof(T) == 8 ? 128 : 64; }
+
 // Register variants: chunks per lane Q (rows up to Q ROWS) and columns per
 // group C.  C is what keeps x within about 64 registers a thread (128 are
 // available) and, at the bench's sizes, takes every column in one pass.

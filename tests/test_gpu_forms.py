@@ -61,3 +61,27 @@ def test_autotune_times_each_launch_once(per_sm, forms):
     ctx = G.Context(2, 3, 3, 4, 4, g=0.4, seed=1)
     assert len(ctx.autotune(ctx.init_configs(n))) == forms
     assert per_sm > 2 or ctx.kernel_name != "gcf::vmc_kernel_grouped4"
+
+
+@pytest.mark.parametrize("prec,cplx,chi", [("fp64", True, 22), ("fp64", False, 43), ("fp32", False, 24)])
+def test_amplitudes_do_not_depend_on_the_batch(prec, cplx, chi):
+    """D_k = 3, bonds beyond the register factorisations in the first two (QR
+    columns of 9 chi rows, Jacobi columns of 3 chi): the same bits alone, among
+    as many chains as there are SMs, among more, and without allocation."""
+    import paper_2503_20566_gb300 as G
+    from paper_2503_20566_gb300.binding import _ptr
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lat, _, vals = oracle_net(10, 7, 2, 6, seed=51, complex_=cplx, precision=prec)
+    ctx = G.Context(2, 10, 7, 6, chi, complex_=cplx, precision=prec, seed=1)
+    ctx.set_tensors(vals)
+    n = sms + 1
+    cfg = ctx.init_configs(n, None, synth.plaquette_powers(52, n, lat.n_plaquettes, 2))
+    ref = ctx.amplitude(cfg)
+    for m in (sms, 3):
+        for a, b in zip(ctx.amplitude(cfg[:m].clone()), ref):
+            assert torch.equal(a, b[:m]), m
+    la, ph = torch.zeros(3, dtype=torch.float64, device="cuda"), torch.zeros(3, dtype=torch.float64, device="cuda")
+    ctx._check(ctx.lib.gcf_amplitude_noalloc(ctx.ctx, 3, _ptr(cfg), _ptr(la), _ptr(ph)), "noalloc")
+    torch.cuda.synchronize()
+    assert torch.equal(la, ref[0][:3]) and torch.equal(ph, ref[1][:3])
