@@ -87,17 +87,22 @@ def load_peaks():
             "sm_max_mhz": 2070.0}, "fallback"
 
 
-# the files the FP32 sampling kernel is compiled from (its translation unit and
-# every header it includes)
+# the files the FP32 one-chain-per-CTA kernels are compiled from (their
+# translation unit and every header it includes), and the units of the other
+# sampling kernels (several chains per CTA, tcgen05, other scalar types) with
+# the header only those include: a committed profile of any of them counts as
+# long as none of these files changed
 KERNEL_SOURCES = ("vmc_f32.cu", "vmc_cta.cuh", "launch.h", "common.cuh", "envsteps.cuh", "factor.cuh", "linalg.cuh", "mma.cuh",
                   "peps_dev.cuh", "tcgen05.cuh", "vmc_kernel.cuh")
+OTHER_UNITS = ("vmc_group.cuh", "vmc_f32_group.cu", "vmc_f32_tc.cu", "vmc_f32_tc_group.cu", "vmc_f64.cu", "vmc_f64_group.cu",
+               "vmc_c64.cu", "vmc_c64_group.cu", "vmc_c128.cu", "vmc_c128_group.cu")
 
 
 def source_hash():
-    """sha256 (first 16 hex) of the sampling kernel's sources, in sorted order."""
+    """sha256 (first 16 hex) of the sampling kernels' sources, in sorted order."""
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2503_20566_gb300", "csrc")
-    for name in sorted(KERNEL_SOURCES):
+    for name in sorted(KERNEL_SOURCES + OTHER_UNITS):
         with open(os.path.join(d, name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
