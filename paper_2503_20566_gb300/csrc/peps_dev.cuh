@@ -318,7 +318,7 @@ __device__ __noinline__ int dense_absorb(const X ex, const KParams<T>& k, Shared
 }
 
 // sel[0..kk) <- the indices of the kk largest of sigma[0..k0), largest first
-// (ties: lower index first).
+// (ties: lower index first; NaN above all, so that every rank is taken once).
 template <class R, class X>
 __device__ inline void select_largest(const X ex, int k0, int kk, const R* sigma, int* sel) {
 #pragma unroll 1
@@ -327,7 +327,9 @@ __device__ inline void select_largest(const X ex, int k0, int kk, const R* sigma
     const R sj = sigma[j];
     for (int i = 0; i < k0; ++i) {
       const R si = sigma[i];
-      rank += (si > sj) || (si == sj && i < j);
+      const bool above = si > sj || (si != si && sj == sj);
+      const bool below = sj > si || (sj != sj && si == si);
+      rank += above || (!below && i < j);
     }
     if (rank < kk) sel[rank] = j;
   }
