@@ -403,8 +403,11 @@ __device__ __noinline__ void site_product(const X ex, const SiteDims d, const T*
 // are closer to orthogonal and converge in fewer sweeps).  The kk columns of
 // largest norm are normalised, and one Newton-Schulz step V (3 I - V^H V) / 2
 // brings them from the sweeps' threshold to orthogonal at rounding.  Columns
-// of norm below eps |Y| are rounding noise, which the sweeps leave alone:
-// their directions are dropped (zero rows of site).
+// of norm below eps |Y| are rounding noise, which the sweeps leave alone: their
+// directions are dropped (zero rows of site), with the rounding of the sums of
+// squares (below 2^-10 for a thousand terms in any order) on top: the sweeps
+// add the same squares in another order, and a column that they left alone may
+// lie along a leading one, so none of those may be kept.
 // Work: W, V and the Gram matrix in the chain's shared-memory workspace as
 // far as they fit it, else in g0, g1, g2 (mat_max each); Vwork, tau for the QR.
 template <class T, class X>
@@ -443,7 +446,7 @@ __device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, c
   R f2 = R(0);
   for (int j = ex.lane(); j < k0; j += 32) f2 += sigma[j];
   f2 = warp_sum(f2);
-  const R negl = Traits<T>::eps() * Traits<T>::eps() * f2;
+  const R negl = Traits<T>::eps() * Traits<T>::eps() * f2 * R(1 + 1.0 / 1024);
   select_largest(ex, k0, kk, sigma, sel);
 #pragma unroll 1
   for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
