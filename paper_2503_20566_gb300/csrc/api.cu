@@ -679,18 +679,6 @@ int cta_block(const gcf_ctx* c, int n_chains) {
   return c->plan.fz_elems > 0 && !c->plan.general && n_chains <= c->sms ? 512 : 256;
 }
 
-int grid_for(gcf_ctx* c, int n_chains) {
-  int per_sm = 1;
-  const int block = cta_block(c, n_chains);
-  switch (c->kind) {
-    case S_F32: per_sm = GCF_TC_CALL(float, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
-    case S_F64: per_sm = GCF_TC_CALL(double, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
-    case S_C64: per_sm = GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
-    default: per_sm = GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem); break;
-  }
-  return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm));
-}
-
 // Resident CTAs per SM of the grouped kernel with W chain groups.
 int grouped_per_sm(const gcf_ctx* c, int W, size_t smem) {
   switch (c->kind) {
@@ -699,6 +687,41 @@ int grouped_per_sm(const gcf_ctx* c, int W, size_t smem) {
     case S_C64: return GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
     default: return GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc_grouped, 128 * W, smem);
   }
+}
+
+// Resident CTAs per SM of vmc_kernel.
+int cta_per_sm(const gcf_ctx* c, int block) {
+  switch (c->kind) {
+    case S_F32: return GCF_TC_CALL(float, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
+    case S_F64: return GCF_TC_CALL(double, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
+    case S_C64: return GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
+    default: return GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
+  }
+}
+
+int grid_for(const gcf_ctx* c, int n_chains) {
+  return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, cta_per_sm(c, cta_block(c, n_chains))));
+}
+
+// A launch of n chains: chains per CTA, CTAs that an SM holds, CTAs when m of
+// them are used.  (Chains do not depend on where they run.)
+struct Shape {
+  int W, per_sm;
+  long long slots(const gcf_ctx* c, int n, int m) const {
+    const long long s = balanced_slots(n, (long long)c->sms * m * W);
+    return (s + W - 1) / W * W;
+  }
+};
+Shape launch_shape(const gcf_ctx* c, int n) {
+  if (!grouped(c)) return {1, std::max(1, cta_per_sm(c, cta_block(c, n)))};
+  const int W = chains_per_cta(c, n);
+  return {W, grouped_per_sm(c, W, W * c->plan.group_smem)};
+}
+// CTAs per SM to use with the scratch that there is: the most that it covers, 0 if none.
+int covered_per_sm(const gcf_ctx* c, const Shape& sh, int n) {
+  int m = sh.per_sm;
+  while (m > 0 && sh.slots(c, n, m) > c->scratch_ctas) --m;
+  return m;
 }
 
 // cudaMalloc that leaves the pointer null when it fails (retry paths free
@@ -710,15 +733,19 @@ bool dalloc(P** p, size_t bytes) {
   return false;
 }
 
-gcf_status ensure_scratch(gcf_ctx* c, long long ctas) {
-  if (ctas <= c->scratch_ctas) return GCF_OK;
+// Scratch for n chains: a full set of slots, and never less than any smaller n
+// takes with one CTA per SM (gcf_sample_batch_async promises those calls).
+gcf_status ensure_scratch(gcf_ctx* c, const Shape& sh, int n) {
+  const long long NG = grouped(c) ? n_groups(c) : 1;
+  const long long below = std::min((n + NG - 1) / NG * NG, c->sms * NG);
+  const long long slots = std::max(below, sh.slots(c, n, sh.per_sm));
+  if (slots <= c->scratch_ctas) return GCF_OK;
   if (c->d_scratch) cudaFree(c->d_scratch);
   c->d_scratch = nullptr;
   c->scratch_ctas = 0;
-  const size_t bytes = (size_t)ctas * c->plan.ws_stride * c->sbytes;
-  cudaError_t e = cudaMalloc(&c->d_scratch, bytes);
-  if (e != cudaSuccess) return fail(c, GCF_ENOMEM, "scratch allocation failed");
-  c->scratch_ctas = ctas;
+  if (!dalloc(&c->d_scratch, (size_t)slots * c->plan.ws_stride * c->sbytes))
+    return fail(c, GCF_ENOMEM, "scratch allocation failed");
+  c->scratch_ctas = slots;
   return GCF_OK;
 }
 
@@ -727,18 +754,14 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
                    int8_t* configs, const gcf_samples* out, int* gauss_count, cudaStream_t stream,
                    bool async) {
   const bool warp = grouped(c);
-  const int W = chains_per_cta(c, n);
-  int grid = 1;
-  if (warp) {
-    const int per_sm = GCF_TC_CALL(T, uses_tc(c), occupancy_vmc_grouped, 128 * W, W * c->plan.group_smem);
-    if (per_sm < 1) return fail(c, GCF_EINVAL, "grouped launch does not fit an SM");
-    const long long slots = balanced_slots(n, (long long)c->sms * per_sm * W);
-    grid = (int)std::max<long long>(1, (slots + W - 1) / W);
-  } else {
-    grid = grid_for(c, n);
+  const Shape sh = launch_shape(c, n);
+  const int W = sh.W;
+  if (sh.per_sm < 1) return fail(c, GCF_EINVAL, "grouped launch does not fit an SM");
+  if (!async) {
+    gcf_status st = ensure_scratch(c, sh, n);
+    if (st != GCF_OK) return st;
   }
-  gcf_status st = ensure_scratch(c, warp ? (long long)grid * W : grid);
-  if (st != GCF_OK) return st;
+  const int grid = (int)(sh.slots(c, n, std::max(1, covered_per_sm(c, sh, n))) / W);
   KParams<T> k = make_params<T>(c);
   if (warp) {
     k.hot_in_smem = c->plan.group_level >= 1;
@@ -1442,21 +1465,10 @@ gcf_status gcf_sample_batch_async(gcf_ctx* c, int n_chains, int n_sweeps, uint64
   DEVICE_TRY(c, "gcf_sample_batch_async");
   cudaStream_t st = stream ? (cudaStream_t)stream : c->stream;
   // scratch must already cover this launch: no allocation here
-  {
-    const bool grp = grouped(c);
-    const int W = chains_per_cta(c, n_chains);
-    long long slots = 1;
-    if (grp) {
-      const int per_sm = grouped_per_sm(c, W, W * c->plan.group_smem);
-      const long long sl = balanced_slots(n_chains, (long long)c->sms * std::max(1, per_sm) * W);
-      slots = (sl + W - 1) / W * W;
-    } else {
-      slots = grid_for(c, n_chains);
-    }
-    if (slots > c->scratch_ctas)
-      return fail(c, GCF_EINVAL, "gcf_sample_batch_async: scratch not yet sized for this many chains; call "
-                                 "gcf_sample_batch with at least as many chains first");
-  }
+  const Shape sh = launch_shape(c, n_chains);
+  if (sh.per_sm >= 1 && covered_per_sm(c, sh, n_chains) < 1)
+    return fail(c, GCF_EINVAL, "gcf_sample_batch_async: scratch not yet sized for this many chains; call "
+                               "gcf_sample_batch with at least as many chains first");
   gcf_samples o{};
   if (out) o = *out;
   int want = (o.log_abs || o.phase ? WANT_AMP : 0) | (o.e_loc ? WANT_ELOC : 0) |
