@@ -4,7 +4,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -91,6 +93,7 @@ struct gcf_ctx {
   int* d_status = nullptr;
   void* d_scratch = nullptr;
   long long scratch_ctas = 0;
+  long long scratch_refused = LLONG_MAX;  // fewest slots that memory had no room for
   // SR work
   SrWork sr{};
   long long sr_ns_cap = 0;
@@ -115,6 +118,7 @@ struct gcf_ctx {
   // context of the call)
   void* multi_arena = nullptr;
   size_t multi_arena_bytes = 0;
+  size_t multi_refused = SIZE_MAX;  // smallest arena that memory had no room for
   void* multi_tab = nullptr;
   size_t multi_tab_bytes = 0;
   int e2e_chains = 0;
@@ -733,20 +737,32 @@ bool dalloc(P** p, size_t bytes) {
   return false;
 }
 
-// Scratch for n chains: a full set of slots, and never less than any smaller n
-// takes with one CTA per SM (gcf_sample_batch_async promises those calls).
-gcf_status ensure_scratch(gcf_ctx* c, const Shape& sh, int n) {
-  const long long NG = grouped(c) ? n_groups(c) : 1;
-  const long long below = std::min((n + NG - 1) / NG * NG, c->sms * NG);
-  const long long slots = std::max(below, sh.slots(c, n, sh.per_sm));
-  if (slots <= c->scratch_ctas) return GCF_OK;
+bool grow_scratch(gcf_ctx* c, long long slots, bool again = false) {
+  if (slots <= c->scratch_ctas) return true;
+  if (slots >= c->scratch_refused && !again) return false;
   if (c->d_scratch) cudaFree(c->d_scratch);
   c->d_scratch = nullptr;
   c->scratch_ctas = 0;
-  if (!dalloc(&c->d_scratch, (size_t)slots * c->plan.ws_stride * c->sbytes))
-    return fail(c, GCF_ENOMEM, "scratch allocation failed");
+  if (!dalloc(&c->d_scratch, (size_t)slots * c->plan.ws_stride * c->sbytes)) {
+    cudaGetLastError();  // a smaller request may follow
+    c->scratch_refused = std::min(c->scratch_refused, slots);
+    return false;
+  }
   c->scratch_ctas = slots;
-  return GCF_OK;
+  return true;
+}
+
+// Scratch for n chains: a full set of slots, and never less than any smaller n
+// takes with one CTA per SM (gcf_sample_batch_async promises those calls).
+// Where memory is short, fewer CTAs per SM: one fits wherever the library ran
+// before a second did.
+gcf_status ensure_scratch(gcf_ctx* c, const Shape& sh, int n) {
+  const long long NG = grouped(c) ? n_groups(c) : 1;
+  const long long below = std::min((n + NG - 1) / NG * NG, c->sms * NG);
+  for (int m = sh.per_sm; m >= 1; --m)
+    if (grow_scratch(c, std::max(below, sh.slots(c, n, m)))) return GCF_OK;
+  if (grow_scratch(c, sh.slots(c, n, 1), true)) return GCF_OK;
+  return fail(c, GCF_ENOMEM, "scratch allocation failed");
 }
 
 template <class T>
@@ -887,16 +903,23 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
   if (per_sm < 1) return fail(c0, GCF_EINVAL, "gcf_sample_multi: the largest context does not fit an SM");
   const int per_cta = block == 512 ? 4 : 1;
   // every resident slot draws from the queue: as many slots as fit, at most
-  // one per chain
-  const long long slots = std::min<long long>(total, (long long)c0->sms * per_sm * per_cta);
-  const long long grid = (slots + per_cta - 1) / per_cta;
-  const size_t arena = (size_t)grid * per_cta * ws * c0->sbytes;
-  if (arena > c0->multi_arena_bytes) {
+  // one per chain; where memory is short, fewer CTAs per SM
+  long long grid = 0;
+  for (int m = per_sm; m >= 1; --m) {
+    const long long slots = std::min<long long>(total, (long long)c0->sms * m * per_cta);
+    grid = (slots + per_cta - 1) / per_cta;
+    const size_t arena = (size_t)grid * per_cta * ws * c0->sbytes;
+    if (arena <= c0->multi_arena_bytes) break;
+    if (m > 1 && arena >= c0->multi_refused) continue;
     if (c0->multi_arena) cudaFree(c0->multi_arena);
-    c0->multi_arena = nullptr;
     c0->multi_arena_bytes = 0;
-    if (cudaMalloc(&c0->multi_arena, arena) != cudaSuccess) return fail(c0, GCF_ENOMEM, "multi-context scratch");
-    c0->multi_arena_bytes = arena;
+    if (dalloc(&c0->multi_arena, arena)) {
+      c0->multi_arena_bytes = arena;
+      break;
+    }
+    cudaGetLastError();
+    c0->multi_refused = std::min(c0->multi_refused, arena);
+    if (m == 1) return fail(c0, GCF_ENOMEM, "multi-context scratch");
   }
   const size_t kb = sizeof(KParams<T>) * n_ctx,
                tb = (kb + 15) / 16 * 16 + sizeof(long long) * (n_ctx + 1) + 16;
