@@ -1024,7 +1024,8 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
       return fail(c, GCF_ENOMEM, "SR vectors");
   }
   if (!c->sr.pbs) {
-    void** grp[4] = {(void**)&c->sr.seg, (void**)&c->sr.seg_v, (void**)&c->sr.seg_b, (void**)&c->sr.pbs};
+    void** grp[5] = {(void**)&c->sr.seg, (void**)&c->sr.part_of, (void**)&c->sr.seg_v, (void**)&c->sr.seg_b,
+                     (void**)&c->sr.pbs};
     for (auto q : grp) {
       if (*q) cudaFree(*q);
       *q = nullptr;
@@ -1037,6 +1038,7 @@ gcf_status ensure_sr(gcf_ctx* c, long long Ns, int n_chains) {
     c->sr.maxnb = maxnb;
     c->sr.n_seg = (int)sv.size();
     if (!dalloc(&c->sr.seg, sizeof(int) * ((size_t)c->n_s * (maxnb + 1) + 1)) ||
+        !dalloc(&c->sr.part_of, sizeof(int) * (size_t)c->n_s * (maxnb + 1)) ||
         !dalloc(&c->sr.seg_v, sizeof(int) * sv.size()) ||
         !dalloc(&c->sr.seg_b, sizeof(int) * sb.size()))
       return fail(c, GCF_ENOMEM, "SR segment tables");
@@ -1189,7 +1191,7 @@ void gcf_destroy(gcf_ctx* c) {
   if (!c) return;
   void* ptrs[] = {c->d_params, c->d_Q, c->d_voff, c->d_vbs, c->d_vnb, c->d_tables, c->d_status,
                   c->d_scratch, c->sr.obar, c->sr.F, c->sr.x, c->sr.r, c->sr.p, c->sr.Ap, c->sr.z, c->sr.dinv,
-                  c->sr.t, c->sr.coef, c->sr.chain_mean, c->sr.scal, c->sr.perm, c->sr.seg, c->sr.count,
+                  c->sr.t, c->sr.coef, c->sr.chain_mean, c->sr.scal, c->sr.perm, c->sr.seg, c->sr.part_of, c->sr.count,
                   c->sr.pbs, c->sr.osort, c->sr.xf, c->sr.coef_f, c->sr.part,
                   c->sr.seg_v, c->sr.seg_b, c->d_cfg, c->d_e,
                   c->d_la, c->d_ph, c->d_bid, c->d_O, c->d_acc, c->vjp_bid, c->vjp_O, c->vjp_coef,

@@ -225,6 +225,10 @@ __global__ void k_update(T* params, const cdouble* x, double cr, double ci, long
 }
 
 // ---------------------------------------------------------------------------
+// Rows of a segment that one warp of k_scatter_warp takes; part[v * (maxnb + 1)
+// + b] counts such parts in the segments of vertex v before block b.
+constexpr int kPartRows = 64;
+
 // Sample order grouped by (vertex, block): for every vertex a stable counting
 // sort of the samples by the block they select.  seg[v * (maxnb + 1) + b] is
 // the start of block b of vertex v inside perm[v * Ns ...]; built once per SR
@@ -232,7 +236,7 @@ __global__ void k_update(T* params, const cdouble* x, double cr, double ci, long
 // block of the vertex come last, behind seg[.. + nb], and set *bad: the step
 // stops before anything is read through such an id.  One CTA per vertex.
 // ---------------------------------------------------------------------------
-__global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm, int* seg, double* bad) {
+__global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm, int* seg, int* part, double* bad) {
   __shared__ int wsum[32];
   __shared__ int base_s;
   const int v = blockIdx.x;
@@ -240,11 +244,15 @@ __global__ void k_sort_by_block(SrGeom g, const int* bids, int maxnb, int* perm,
   const long long Ns = g.Ns;
   int* pv = perm + (long long)v * Ns;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int prev = 0, parts = 0;  // thread 0
   if (threadIdx.x == 0) base_s = 0;
   __syncthreads();
   for (int b = 0; b <= nb; ++b) {
     if (threadIdx.x == 0) {
       seg[v * (maxnb + 1) + b] = base_s;
+      parts += (base_s - prev + kPartRows - 1) / kPartRows;
+      part[v * (maxnb + 1) + b] = parts;
+      prev = base_s;
       if (b == nb && base_s < Ns) *bad = 1.0;
     }
     __syncthreads();
@@ -303,7 +311,7 @@ __global__ void k_sort_count(SrGeom g, const int* bids, int maxnb, int n_chunk, 
     count[((long long)v * (maxnb + 1) + i) * n_chunk + blockIdx.x] = t;
   }
 }
-__global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* seg, double* bad) {
+__global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* seg, int* part, double* bad) {
   __shared__ int tot[kSortBlocks + 1];
   const int v = blockIdx.x, nb = g.vnb[v] + 1, lane = threadIdx.x & 31;
   int* cv = count + (long long)v * (maxnb + 1) * n_chunk;
@@ -315,12 +323,14 @@ __global__ void k_sort_scan(SrGeom g, int maxnb, int n_chunk, int* count, int* s
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int acc = 0;
+    int acc = 0, parts = 0;
     for (int b = 0; b < nb; ++b) {
       const int t = tot[b];
       tot[b] = acc;
       seg[v * (maxnb + 1) + b] = acc;
+      part[v * (maxnb + 1) + b] = parts;
       acc += t;
+      parts += (t + kPartRows - 1) / kPartRows;
       if (b == nb - 1 && t > 0) *bad = 1.0;
     }
   }
@@ -585,21 +595,29 @@ __global__ void k_scatter_sorted(SrGeom g, const int* perm, const int* seg, int 
   }
 }
 
-// k_scatter_sorted with a warp per segment, for short segments of blocks of at
+// k_scatter_sorted with a warp per kPartRows rows of a segment, for blocks of at
 // most 32 entries: lanes take 32 / bs rows at a time (a CTA per segment of 38
-// rows: 80 us at 1024 complex samples of 16x16 Z3).
+// rows: 80 us at 1024 complex samples of 16x16 Z3).  Segments are split by their
+// own length: near a ground state one block of a vertex holds most samples (16000
+// complex samples of 8x8 Z4 with matter, nine in ten on one block, 20 CG steps:
+// 92 ms with a warp for a whole segment, 28 with a CTA, 5.7 in parts).  Warp w of
+// vertex blockIdx.y finds its segment in the table of parts.
 template <class T, bool CONJ, bool CPLX, bool SQ>
-__global__ void k_scatter_warp(SrGeom g, const int* perm, const int* seg, int maxnb, int n_seg, const T* osort,
-                               const long long* pbs, const cdouble* coef, cdouble* out, const int* seg_v,
-                               const int* seg_b) {
+__global__ void k_scatter_warp(SrGeom g, const int* perm, const int* seg, const int* part_of, int maxnb, const T* osort,
+                               const long long* pbs, const cdouble* coef, cdouble* out) {
   using P = typename PartialOf<T>::type;
   const int lane = threadIdx.x & 31;
-  const int sid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (sid >= n_seg) return;
-  const int v = seg_v[sid], b = seg_b[sid];
+  const int v = blockIdx.y, w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nb = g.vnb[v];
+  const int* pt = part_of + v * (maxnb + 1);
+  if (w >= pt[nb]) return;
+  int b = 0;  // the last segment whose parts start at or before w
+  for (int hi = nb; hi - b > 1;) {
+    const int mid = (b + hi) >> 1;
+    if (pt[mid] <= w) b = mid;
+    else hi = mid;
+  }
   const int bs = g.vbs[v], rpw = 32 / bs;
-  const int s0 = seg[v * (maxnb + 1) + b], s1 = seg[v * (maxnb + 1) + b + 1];
-  if (s0 >= s1) return;
+  const int s0 = seg[v * (maxnb + 1) + b] + (w - pt[b]) * kPartRows, s1 = min(seg[v * (maxnb + 1) + b + 1], s0 + kPartRows);
   const int* pv = perm + (long long)v * g.Ns;
   const T* rows = osort + g.Ns * pbs[v];
   const int rr = lane / bs, e = lane - rr * bs;
@@ -767,16 +785,13 @@ static cudaError_t scatter(const SrGeom& g, const SrWork& w, const T* O, const c
     }
   }
   if (g.D4 <= 32 && per_seg < 256) {
-    const int blocks = nblk((long long)w.n_seg * 32, 256);
+    const dim3 blocks((unsigned)nblk((g.Ns / kPartRows + w.maxnb) * 32, 256), (unsigned)g.n_s);
     if (sq)
-      k_scatter_warp<T, false, C, true><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
-                                                                out, w.seg_v, w.seg_b);
+      k_scatter_warp<T, false, C, true><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.part_of, w.maxnb, os, w.pbs, coef, out);
     else if (conj)
-      k_scatter_warp<T, true, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
-                                                                out, w.seg_v, w.seg_b);
+      k_scatter_warp<T, true, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.part_of, w.maxnb, os, w.pbs, coef, out);
     else
-      k_scatter_warp<T, false, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.maxnb, w.n_seg, os, w.pbs, coef,
-                                                                 out, w.seg_v, w.seg_b);
+      k_scatter_warp<T, false, C, false><<<blocks, 256, 0, st>>>(g, w.perm, w.seg, w.part_of, w.maxnb, os, w.pbs, coef, out);
     ++*launches;
     return cudaGetLastError();
   }
@@ -843,11 +858,11 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
     const dim3 grid((unsigned)n_chunk, (unsigned)g.n_s);
     const size_t smem = sizeof(int) * 32 * (w.maxnb + 1);
     k_sort_count<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count);
-    k_sort_scan<<<g.n_s, 256, 0, st>>>(g, w.maxnb, n_chunk, w.count, w.seg, w.scal + 3);
+    k_sort_scan<<<g.n_s, 256, 0, st>>>(g, w.maxnb, n_chunk, w.count, w.seg, w.part_of, w.scal + 3);
     k_sort_place<<<grid, 1024, smem, st>>>(g, bids, w.maxnb, n_chunk, w.count, w.perm);
     *launches += 3;
   } else {
-    k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg, w.scal + 3);
+    k_sort_by_block<<<g.n_s, 1024, 0, st>>>(g, bids, w.maxnb, w.perm, w.seg, w.part_of, w.scal + 3);
     ++*launches;
   }
   // O in segment order, streamed by every scatter of this step

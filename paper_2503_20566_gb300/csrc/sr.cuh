@@ -31,6 +31,7 @@ struct SrWork {
   // sample order grouped by (vertex, block)
   int* perm;      // [n_s * Ns]
   int* seg;       // [n_s * (maxnb + 1)]
+  int* part_of;   // [n_s * (maxnb + 1)] parts of the segments before each block (k_scatter_warp)
   int* count;     // [n_s * (maxnb + 1) * chunks of 1024 samples] of the chunked sort; null: the other sort
   int* seg_v;     // [n_seg] vertex of segment
   int* seg_b;     // [n_seg] block of segment

@@ -43,11 +43,14 @@ def _samples(bid, O, E):
     (5, 3, 10, 600, "fp32", False, True), (5, 3, 10, 1300, "fp64", True, True), (2, 3, 6, 1500, "fp32", False, False),
     (2, 3, 6, 1025, "fp32", True, False), (2, 3, 6, 1500, "fp64", False, False), (3, 2, 3, 2100, "fp32", False, False)])
 def test_sr_update_many_blocks_and_odd_sizes(N, L, D, n, prec, cplx, matter):
-    ctx, nb, bs, bid, O, E = _problem(N, L, D, n, prec, cplx, matter)
-    shift, lr = 0.1, 0.5
+    _check(*_problem(N, L, D, n, prec, cplx, matter), prec)
+
+
+def _check(ctx, nb, bs, bid, O, E, prec):
+    shift, lr, n, cplx = 0.1, 0.5, len(E), np.iscomplexobj(O)
     off = np.concatenate([[0], np.cumsum([a * b for a, b in zip(nb, bs)])])
     c = np.zeros((n, off[-1]), np.complex128 if cplx else np.float64)
-    for v in range(L * L):
+    for v in range(len(nb)):
         np.put_along_axis(c, off[v] + bid[:, v, None] * bs[v] + np.arange(bs[v]), O[:, v, :bs[v]].astype(c.dtype), 1)
     F = c.conj().T @ (E - E.mean()) / n
     c -= c.mean(0)
@@ -61,6 +64,18 @@ def test_sr_update_many_blocks_and_odd_sizes(N, L, D, n, prec, cplx, matter):
     eps = 2.0 ** -23 if prec == "fp32" else 1e-15
     tol = (1e-4 if prec == "fp32" else 1e-9) * np.abs(x).max() + eps * np.abs(before).max() / lr
     assert np.abs(got - x).max() <= tol, (np.abs(got - x).max(), tol)
+
+
+@pytest.mark.parametrize("N,D,prec,cplx", [(3, 6, "fp32", True), (3, 6, "fp64", False), (3, 3, "fp32", False)])
+def test_sr_update_with_most_samples_on_one_block(N, D, prec, cplx):
+    """Short segments on average, long ones among them: warps take 64 rows each,
+    so segments of 0, 1, 63, 64, 65, 128 and about a thousand rows meet."""
+    ctx, nb, bs, bid, O, E = _problem(N, 3, D, 1400, prec, cplx, False)
+    for v in range(9):
+        lens = [0, 1, 63, 64, 65, 128][: min(6, nb[v] - 1)]
+        bid[:, v] = np.random.default_rng(v).permutation(np.concatenate([np.repeat(np.arange(len(lens)), lens),
+                                                                         np.full(1400 - sum(lens), nb[v] - 1)]))
+    _check(ctx, nb, bs, bid, O, E, prec)
 
 
 @pytest.mark.parametrize("N,D,matter,prec,cplx", [(2, 4, False, "fp32", False), (5, 10, True, "fp32", False), (3, 9, False, "fp64", True)])
