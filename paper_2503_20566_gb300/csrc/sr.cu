@@ -411,10 +411,13 @@ __global__ void k_gather2(SrGeom g, const int* bids, const T* O, const cdouble* 
 // The same product with each sample's O row (n_s x D4 storage scalars,
 // contiguous) read by the whole warp in 16-byte vectors; needs D4 a multiple
 // of VE = 16 / sizeof(T).  Per-vector partials in the storage precision,
-// then FP64.  BLK: by a block of 256 instead of a warp, for few samples (1024
-// warps leave the chip idle: 74 us at 1024 complex samples of 16x16, D_k = 2;
-// the floor of 34 MB is 5).
-constexpr long long kBlockGatherBelow = 16384;  // samples: 152 SMs x 64 warps hold about 10000
+// then FP64.  BLK: by a block of 256 instead of a warp, for few samples of long
+// rows (1024 warps leave the chip idle: 74 us at 1024 complex samples of 16x16,
+// D_k = 2; the floor of 34 MB is 5).  The line, samples = twice the vectors of a
+// row, is where the two met on 2x2 to 16x16 (steps of 20 iterations, block /
+// warp: 16x16 complex 0.58 at 128 samples, 0.97 at 4096, 1.05 at 24000; 8x8
+// complex 0.85, 1.11 and 1.20; 3x3 real 1.00, 1.14 and 1.66).
+inline bool gather_by_block(long long samples, long long vectors) { return samples <= 2 * vectors; }
 template <class T, bool CPLX, bool BLK>
 __global__ void k_gather_vec(SrGeom g, const int* bids, const T* O, const cdouble* x, cdouble* t) {
   using P = typename PartialOf<T>::type;
@@ -925,7 +928,7 @@ cudaError_t sr_solve_update(const SrGeom& g, SrWork& w, const double* e_loc, con
   bool converged = !(fnorm > 0.0);
   bool quad = false;
   if constexpr (std::is_same<T, float>::value) quad = vec_ok && w.all_bs4 && d4_shift >= 2;
-  const bool blk = Ns < kBlockGatherBelow;
+  const bool blk = gather_by_block(Ns, (long long)g.n_s * g.D4 * (long long)sizeof(T) / 16);
   const int vgrid = (int)std::min<long long>(nblk(Np, 256), 1024);
   if (quad && !converged && max_iter > 0) {
     k_real_to_f32<<<nblk(Np, 256), 256, 0, st>>>(w.p, Np, w.xf);

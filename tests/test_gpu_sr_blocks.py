@@ -41,7 +41,10 @@ def _samples(bid, O, E):
 
 @pytest.mark.parametrize("N,L,D,n,prec,cplx,matter", [
     (5, 3, 10, 600, "fp32", False, True), (5, 3, 10, 1300, "fp64", True, True), (2, 3, 6, 1500, "fp32", False, False),
-    (2, 3, 6, 1025, "fp32", True, False), (2, 3, 6, 1500, "fp64", False, False), (3, 2, 3, 2100, "fp32", False, False)])
+    (2, 3, 6, 1025, "fp32", True, False), (2, 3, 6, 1500, "fp64", False, False), (3, 2, 3, 2100, "fp32", False, False),
+    # a block gathers a sample up to twice as many samples as a row has vectors (36 and 72 here), a warp beyond
+    (2, 3, 4, 72, "fp32", False, False), (2, 3, 4, 73, "fp32", False, False), (2, 3, 4, 144, "fp32", True, False),
+    (2, 3, 4, 145, "fp32", True, False)])
 def test_sr_update_many_blocks_and_odd_sizes(N, L, D, n, prec, cplx, matter):
     _check(*_problem(N, L, D, n, prec, cplx, matter), prec)
 
