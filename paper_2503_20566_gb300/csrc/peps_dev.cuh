@@ -1,5 +1,5 @@
 // Device layer of the GCF-PEPS contraction: sector gather (Sec. S-2, Eq. S5),
-// boundary-MPS row absorption with QR / LQ / truncated-SVD compression, and
+// boundary-MPS row absorption with QR / truncated-SVD compression, and
 // the environment steps of the 4-layer strip (plaquette and vertical-hop
 // ratios) and of the 3-layer row (gradient and horizontal-hop ratios).
 //
@@ -238,8 +238,8 @@ __device__ __noinline__ void cta_dot(const X ex, const T* A, const T* B, int n, 
 // exact MPS whose sites left of m = floor(L/2) are identity isometries
 // M[a][i][a*p + i], whose sites right of m are identity isometries
 // M[i*p^(L-1-c) + b][i][b], and whose site m holds the normalised dense state
-// v[(u_0..u_{m-1})][u_m][(u_{m+1}..u_{L-1})].  It is the same state the QR /
-// LQ sweep produces, in a different gauge.  The dense state is obtained by
+// v[(u_0..u_{m-1})][u_m][(u_{m+1}..u_{L-1})].  It is the same state the sweeps
+// of the general path produce, in a different gauge.  The dense state is obtained by
 // contracting the input MPS to a vector and applying the row MPO site by site.
 // Returns the binary exponent e of the scale (state = 2^e * output).
 // ---------------------------------------------------------------------------
@@ -513,10 +513,16 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
 
   // General path.  Z_c (absorbed sites) right of cL; then a QR sweep from the
   // left over the bonds that must shrink (all bonds if the step truncates),
-  // then an LQ / truncated-SVD sweep from the right over the bonds that must
-  // shrink; sites in between are the absorbed tensors with the carries
-  // multiplied in.  Without truncation this reaches the exact state with the
-  // step's bond dimensions; with truncation it is the full canonical sweep.
+  // then a sweep from the right over the bonds that must shrink (truncated SVD,
+  // or the identity where the outer dimensions fit); sites in between are the
+  // absorbed tensors with the carries multiplied in.  Without truncation this
+  // reaches the exact state with the step's bond dimensions; with truncation it
+  // is the full canonical sweep.  Where no bond shrinks from the left (cL = 0:
+  // the first rows of a lattice) every site is a Z_c, and one that needs no
+  // carry either goes to the output as it is: those steps are short, and the
+  // code of a longer way through them costs more than their work (16 amplitudes on
+  // 4x4, D_k = 3, chi = 9, complex FP32: 166 -> 156 us; 608 FP32 chains of 4x4
+  // with bosons, four sweeps: 6.13 -> 5.80 ms).
   if (ex.tid() == 0) {
     int any_svd = 0;
     for (int c = 1; c < Lx; ++c) any_svd |= svd[c];
@@ -541,7 +547,7 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   T* Y = ws + k.o_W1;
   T* Lc = ws + k.o_W4;
   T* Vw = ws + k.o_W2;
-  for (int c = cL + 1; c < Lx; ++c) {
+  for (int c = cL ? cL + 1 : 0; c < Lx; ++c) {
     const int a = bdi[c], b = bdi[c + 1];
     const int l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
     const T* M = mps_in + sh.bd_off[c];
@@ -568,7 +574,7 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   ex.sync();
   int Rrows = 1, ldr = 4, ldxb = 4;
   T* fz = (T*)g_fz[ex.slot()];
-  for (int c = 0; c <= cL; ++c) {
+  for (int c = 0; c <= cL && cL; ++c) {
     const int cols = sh.ab[c + 1], rows = Rrows * pout, ldx = pad4(rows);
     const int nb = bdi[c + 1], l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
     // X ((Rrows pout) x (b, r)) = sum R[.][(a l)] M[a][d][b] W[l][r][d][u], the
@@ -609,30 +615,39 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
     const int cur = (c < cL) ? qr[c] : (c == cL ? Rrows : sh.ab[c]);
     const int rd = (c < cL) ? qr[c + 1] : sh.ab[c + 1];
     const int n = ident ? rd : kc, yc = pout * n, ldy = pad4(cur), rows = cur * pout;
+    const bool from_x = c == cL && cL, shrinks = c >= 1 && (svd[c] || bdo[c] < cur);
+    const T* S = from_x ? Xb : Z + sh.zoff[c];
+    T* site = mout + sh.bd_off2[c];
+    if (ident && c >= cL && !shrinks) {
+      // the absorbed site as it is
+#pragma unroll 1
+      for (int idx = ex.tid(); idx < rows * n; idx += ex.size())
+        site[idx] = from_x ? S[(idx % n) * ldxb + idx / n] : S[idx];
+      ex.sync();
+      logs += rescale(ex, site, rows * n);
+      continue;
+    }
     if (c < cL && rows > rd) {
       const T* V = Qs + sh.qoff[c];
       const int ldv = pad4(rows);
       apply_q<T>(ex, rows, rd, V, ldv, V + ldv * rd, ident ? (const T*)nullptr : Lc, ldl, n, pout, Y, ldy, M1);
     } else if (c < cL || ident) {
       // identity isometry (Y = the carry) or identity carry (Y = the site)
-      const T* S = c == cL ? Xb : Z + sh.zoff[c];
 #pragma unroll 1
       for (int idx = ex.tid(); idx < rows * n; idx += ex.size()) {
         const int m = idx / rows, q = idx - (idx / rows) * rows;
         const int i = q / pout, u = q - (q / pout) * pout;
         T v;
         if (c < cL) v = ident ? (q == m ? one<T>() : zero<T>()) : Lc[m * ldl + q];
-        else v = c == cL ? S[m * ldxb + q] : S[q * rd + m];
+        else v = from_x ? S[m * ldxb + q] : S[q * rd + m];
         Y[(u * n + m) * ldy + i] = v;
       }
       ex.sync();
     } else {
-      const T* S = c == cL ? Xb : Z + sh.zoff[c];
-      cta_gemm_out<T>(ex, rows, n, rd, S, {1, c == cL ? 1 : rd, 0}, c == cL ? ldxb : 1, Lc, 1, ldl,
+      cta_gemm_out<T>(ex, rows, n, rd, S, {1, from_x ? 1 : rd, 0}, from_x ? ldxb : 1, Lc, 1, ldl,
                       OutMap<T>{Y, {pout, 1, n * ldy}, n, 0, ldy});
     }
-    T* site = mout + sh.bd_off2[c];
-    if (c >= 1 && (svd[c] || bdo[c] < cur)) {
+    if (shrinks) {
       const int kk = bdo[c];
       if (!svd[c]) {
         // yc = kk columns already fit the bond: the identity is the isometry
