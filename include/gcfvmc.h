@@ -386,7 +386,8 @@ gcf_status gcf_set_svd_sweeps(gcf_ctx* ctx, int max_sweeps);
  * (implementation choice; no counterpart in the paper): 0 = configuration
  * only, 1 = + hot buffers (network boxes, proposals, current environments,
  * GEMM temporaries), 2 = + the staged boundary-MPS rows of the current pass,
- * 3 = + the right environments of the pass. */
+ * 3 = + the right environments of the pass.  One chain per CTA: the level of
+ * calls with more chains than SMs; others may take a larger one. */
 int gcf_smem_level(const gcf_ctx* ctx);
 
 /* Autotuner (implementation choice; no counterpart in the paper): times every

@@ -44,7 +44,7 @@ struct Plan {
   size_t dyn_smem = 0;
   // shared-memory placement levels of the two kernel forms (see plan_group)
   long long hot_base_elems = 0, hot_mps_elems = 0, hot_all_elems = 0;
-  int cta_level = 0, group_level = 0;
+  int cta_level = 0, cta_level_few = 0, group_level = 0;  // few: at most one chain per SM
   size_t group_smem = 0;
   // BF16 form of real chains: bytes of the tcgen05 operand staging area of
   // one chain (0: the tensor-core GEMMs of that form stay on mma.sync)
@@ -341,7 +341,7 @@ void set_form(gcf_ctx* c, int exec, int level) {
     p.group_level = level;
     p.group_smem = group_smem_bytes(p, level, c->sbytes);
   } else {
-    p.cta_level = level;
+    p.cta_level = p.cta_level_few = level;
     p.hot_elems = p.level_elems(level);
     p.dyn_smem = cta_smem_bytes(p, level, c->sbytes);
   }
@@ -571,12 +571,16 @@ void build_plan(gcf_ctx* c) {
     if (Nmax <= 128) p.tc_bytes = (tc_stage_bytes(Nmax, Kmax) + 15) / 16 * 16;
   }
   // one chain per CTA: the largest level that keeps two CTAs on an SM (113 KB
-  // each, 16 KB of it static)
-  const size_t budget = 96 * 1024;
-  p.cta_level = 0;
-  for (int lv = 1; lv <= 3; ++lv)
-    if (cta_smem_bytes(p, lv, c->sbytes) <= budget) p.cta_level = lv;
-  if (const char* e = std::getenv("GCFVMC_SMEM_CTA")) p.cta_level = std::max(0, std::min(3, std::atoi(e)));
+  // each, 16 KB of it static); with at most one chain per SM there is no second
+  // CTA to make room for (E_loc 10x3, chi = 32, complex FP64, 16 chains: 1.46 ms
+  // at level 2, 1.18 at level 3 with 97 KB)
+  p.cta_level = p.cta_level_few = 0;
+  for (int lv = 1; lv <= 3; ++lv) {
+    if (cta_smem_bytes(p, lv, c->sbytes) <= 96 * 1024) p.cta_level = lv;
+    if (cta_smem_bytes(p, lv, c->sbytes) <= 100 * 1024) p.cta_level_few = lv;
+  }
+  if (const char* e = std::getenv("GCFVMC_SMEM_CTA"))
+    p.cta_level = p.cta_level_few = std::max(0, std::min(3, std::atoi(e)));
   p.hot_elems = p.level_elems(p.cta_level);
   p.dyn_smem = cta_smem_bytes(p, p.cta_level, c->sbytes);
   plan_group(c);
@@ -693,18 +697,18 @@ int grouped_per_sm(const gcf_ctx* c, int W, size_t smem) {
   }
 }
 
-// Resident CTAs per SM of vmc_kernel.
-int cta_per_sm(const gcf_ctx* c, int block) {
-  switch (c->kind) {
-    case S_F32: return GCF_TC_CALL(float, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
-    case S_F64: return GCF_TC_CALL(double, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
-    case S_C64: return GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
-    default: return GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc, block, c->plan.dyn_smem);
-  }
-}
+// Shared-memory level and dynamic shared memory of vmc_kernel for n chains.
+int cta_level(const gcf_ctx* c, int n) { return n <= c->sms ? c->plan.cta_level_few : c->plan.cta_level; }
+size_t cta_smem(const gcf_ctx* c, int n) { return cta_smem_bytes(c->plan, cta_level(c, n), c->sbytes); }
 
-int grid_for(const gcf_ctx* c, int n_chains) {
-  return (int)balanced_slots(n_chains, (long long)c->sms * std::max(1, cta_per_sm(c, cta_block(c, n_chains))));
+// Resident CTAs per SM of vmc_kernel.
+int cta_per_sm(const gcf_ctx* c, int block, size_t smem) {
+  switch (c->kind) {
+    case S_F32: return GCF_TC_CALL(float, uses_tc(c), occupancy_vmc, block, smem);
+    case S_F64: return GCF_TC_CALL(double, uses_tc(c), occupancy_vmc, block, smem);
+    case S_C64: return GCF_TC_CALL(cfloat, uses_tc(c), occupancy_vmc, block, smem);
+    default: return GCF_TC_CALL(cdouble, uses_tc(c), occupancy_vmc, block, smem);
+  }
 }
 
 // A launch of n chains: chains per CTA, CTAs that an SM holds, CTAs when m of
@@ -717,7 +721,7 @@ struct Shape {
   }
 };
 Shape launch_shape(const gcf_ctx* c, int n) {
-  if (!grouped(c)) return {1, std::max(1, cta_per_sm(c, cta_block(c, n)))};
+  if (!grouped(c)) return {1, std::max(1, cta_per_sm(c, cta_block(c, n), cta_smem(c, n)))};
   const int W = chains_per_cta(c, n);
   return {W, grouped_per_sm(c, W, W * c->plan.group_smem)};
 }
@@ -785,6 +789,13 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
     k.renv_in_smem = c->plan.group_level >= 3;
     k.tc_off = (long long)group_tc_off(c->plan, c->plan.group_level, c->sbytes);
     k.fz_off = (long long)group_fz_off(c->plan, c->plan.group_level, c->sbytes);
+  } else {
+    const int lv = cta_level(c, n);
+    k.hot_in_smem = lv >= 1;
+    k.mps_in_smem = lv >= 2;
+    k.renv_in_smem = lv >= 3;
+    k.tc_off = (long long)cta_tc_off(c->plan, lv, c->sbytes);
+    k.fz_off = (long long)cta_fz_off(c->plan, lv, c->sbytes);
   }
   if (warp && W == 1) k.lockstep = 0;
   k.n_chains = n; k.n_sweeps = n_sweeps; k.mode = mode; k.want = want; k.seed = seed;
@@ -798,7 +809,7 @@ gcf_status run_vmc(gcf_ctx* c, int mode, int want, int n, int n_sweeps, uint64_t
   if (warp)
     CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc_grouped, k, grid, 128 * W, W * c->plan.group_smem, stream));
   else
-    CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc, k, grid, cta_block(c, n), c->plan.dyn_smem, stream));
+    CUDA_TRY(c, GCF_TC_CALL(T, uses_tc(c), launch_vmc, k, grid, cta_block(c, n), cta_smem(c, n), stream));
   c->launches += 1;
   c->last_chains = warp ? W : 1;
   if (async) return GCF_OK;
@@ -1664,7 +1675,7 @@ gcf_status amplitude_noalloc_impl(gcf_ctx* c, int n, const int8_t* configs, doub
                   per_cta);
     return fail(c, GCF_EINVAL, msg);
   }
-  const int grid = (int)std::max<long long>(1, std::min<long long>(fit, grid_for(c, n)));
+  const int grid = (int)std::max<long long>(1, std::min<long long>(fit, balanced_slots(n, (long long)c->sms * std::max(1, cta_per_sm(c, 256, c->plan.dyn_smem)))));
   KParams<T> k = make_params<T>(c);
   k.scratch = (T*)scratch;
   k.status = status;
