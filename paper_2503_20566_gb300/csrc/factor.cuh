@@ -142,7 +142,7 @@ __device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, bool
   const R xn2 = sum8(p0 + p1);
   al = sum8s(al);
   T t, sc, beta;
-  householder_fast(al, xn2, t, sc, beta);
+  householder(al, xn2, t, sc, beta);
   if (own) {
 #pragma unroll
     for (int q = 0; q < Q; ++q) {

@@ -141,14 +141,8 @@ __device__ inline void householder(T alpha, typename Traits<T>::R xn2, T& tau, T
   beta = make_scalar<T>(b, R(0));
 }
 
-// Reciprocal (to rounding, without the special cases of a division), and
-// square root, reciprocal and reciprocal square root in which a few units in
-// the last place do not matter (FP32: the hardware's; FP64: exact).
-__device__ __forceinline__ float rcp1(float x) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return fmaf(r, fmaf(-x, r, 1.f), r);
-}
+// Reciprocal, square root and reciprocal square root of the rotation angles, in
+// which a few units in the last place do not matter (FP32: the hardware's; FP64: exact).
 __device__ __forceinline__ float jrcpa(float x) {
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -167,31 +161,6 @@ __device__ __forceinline__ float jrsqrt1(float x) {
 __device__ __forceinline__ double jrcpa(double x) { return 1.0 / x; }
 __device__ __forceinline__ double jsqrta(double x) { return sqrt(x); }
 __device__ __forceinline__ double jrsqrt1(double x) { return 1.0 / sqrt(x); }
-
-// householder() with the two divisions replaced by independent reciprocals
-// where the column's norm is far from the range's ends (FP32): a reflector is
-// the longest link of a QR step's chain.
-template <class T>
-__device__ __forceinline__ void householder_fast(T alpha, typename Traits<T>::R xn2, T& tau, T& scal, T& beta) {
-  if constexpr (sizeof(typename Traits<T>::R) == 4) {
-    const float ar = re(alpha), ai = im(alpha);
-    const float s2 = fmaf(ar, ar, fmaf(ai, ai, xn2));
-    if (s2 > 1e-30f && s2 < 1e30f && (xn2 > 0.f || ai != 0.f)) {
-      const float b = ar >= 0.f ? -sqrtf(s2) : sqrtf(s2);
-      const float ib = rcp1(b), dr = ar - b;
-      if constexpr (Traits<T>::cplx) {
-        const float id2 = rcp1(fmaf(dr, dr, ai * ai));
-        scal = make_scalar<T>(dr * id2, -ai * id2);
-      } else {
-        scal = rcp1(dr);
-      }
-      tau = make_scalar<T>(-dr * ib, -ai * ib);
-      beta = make_scalar<T>(b, 0.f);
-      return;
-    }
-  }
-  householder(alpha, xn2, tau, scal, beta);
-}
 
 // Sum of v over the L consecutive lanes (L a power of two <= 32, aligned)
 // that share a column pair; every lane of the warp must call it.
