@@ -167,7 +167,12 @@ __device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, bool
 // in chunks of 16 bytes over the lanes (at most Q chunks a lane).  Reflectors
 // of earlier passes come from V.  Per step one barrier: the group that
 // holds column j + 1 updates it first and publishes its reflector (two
-// buffers in vb) while the others are still updating.
+// buffers in vb) while the others are still updating.  Except in real FP32 a warp
+// skips a slot whose four columns are finished or beyond the matrix (SKIP): FP64
+// and complex multiply-adds are what a step waits for (amplitudes 8x4, D_k = 3,
+// chi = 22, FP64, 16 chains 6.50 -> 5.86 ms; sampling 10x10 chi = 16 FP64 69.7 ->
+// 64.6 ms), in real FP32 the branches cost more (three boson lattices, 5472
+// chains: 15.06 s without, 15.19 s with).
 // Outputs: V (explicit reflector columns: zero above, 1 on the diagonal) and
 // tau when V is set; the rows 0 .. k - 1 (k = min(m, n)) of R either as
 // column-major Rt (leading dimension ldr) or, TRANS, as the columns of
@@ -178,6 +183,8 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
   const int k = min(m, n), mp = (m + E - 1) / E * E, ldb = (m + 8 * E - 1) / (8 * E) * (8 * E), nq = ldb / (8 * E);
+  constexpr bool SKIP = sizeof(T) > 4;
+  const int w4 = ex.warp() << 2;  // the warp's first group
   T* tb = vb + 2 * ldb;
   T x[C][Q * E];
 #pragma unroll
@@ -201,7 +208,7 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
     const T f = conjg(tau[j]);
 #pragma unroll
     for (int s = 0; s < C; ++s)
-      if (c0 + s * ngrp < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
+      if (c0 + s * ngrp + w4 < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
   }
   if (c0 < k && ex.warp() == 0)
     make_reflector<T, Q>(x[0], c0, nq, li, grp == 0, vb + (c0 & 1) * ldb, tb + (c0 & 1));
@@ -216,7 +223,9 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
       const T f = conjg(tb[j & 1]);
       const int q0 = j / (8 * E);
       if (ex.tid() == 0 && V) tau[j] = tb[j & 1];
+      const bool cur = !SKIP || (w4 + 3 > jj && c0 + s * ngrp + w4 < n);  // columns of slot s left to this warp
       if constexpr (C > 1) {
+        if (SKIP && !cur && !(s + 1 < C && c0 + (s + 1) * ngrp + w4 < n)) continue;
         T vr[Q * E];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -226,13 +235,14 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
             for (int e = 0; e < E; ++e) vr[q * E + e] = zero<T>();
           }
         }
-        reflect_col<T, Q>(x[s], vr, grp > jj ? f : zero<T>(), q0);
+        if (cur) reflect_col<T, Q>(x[s], vr, grp > jj ? f : zero<T>(), q0);
         if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
           make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
 #pragma unroll
         for (int s2 = s + 1; s2 < C; ++s2)
-          if (c0 + s2 * ngrp < n) reflect_col<T, Q>(x[s2], vr, f, q0);
+          if (c0 + s2 * ngrp + (SKIP ? w4 : 0) < n) reflect_col<T, Q>(x[s2], vr, f, q0);
       } else {
+        if (!cur) continue;
         reflect_col_mem<T, Q>(x[s], v, li, grp > jj ? f : zero<T>(), q0, ldb);
         if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
           make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
@@ -281,7 +291,8 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
                                           int ldl, int nc, int c0, int pout, T* Y, int ldy) {
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
-  const int mp = (m + E - 1) / E * E;
+  const int mp = (m + E - 1) / E * E, w4 = ex.warp() << 2;
+  if (c0 + w4 >= nc) return;  // no column for this warp
   T x[C][Q * E];
 #pragma unroll
   for (int s = 0; s < C; ++s) {
@@ -328,7 +339,7 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
         const int q0 = j / (8 * E);
 #pragma unroll
         for (int s = 0; s < C; ++s)
-          if (s == 0 || c0 + s * ngrp < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0);
+          if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0);
         fetch(vr[a], j - AHEAD);
         fr[a] = tau[max(j - AHEAD, 0)];
       }
@@ -339,7 +350,7 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
       const T f = tau[j];
 #pragma unroll
       for (int s = 0; s < C; ++s)
-        if (s == 0 || c0 + s * ngrp < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
+        if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
     }
   }
 #pragma unroll
