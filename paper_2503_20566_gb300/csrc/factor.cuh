@@ -162,8 +162,8 @@ __device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, bool
   __syncwarp();
 }
 
-// One register pass of the Householder QR of A (m x n, column-major): columns
-// c0 .. c0 + groups C - 1, a column per group of 8 lanes and slot, its rows
+// Householder QR of A (m x n, column-major) in register passes: columns c0 ..
+// c0 + groups C - 1, a column per group of 8 lanes and slot, its rows
 // in chunks of 16 bytes over the lanes (at most Q chunks a lane).  Reflectors
 // of earlier passes come from V.  Per step one barrier: the group that
 // holds column j + 1 updates it first and publishes its reflector (two
@@ -178,7 +178,7 @@ __device__ __forceinline__ void make_reflector(T* x, int j, int nq, int li, bool
 // column-major Rt (leading dimension ldr) or, TRANS, as the columns of
 // W = R^H: W[c + i ldr] = conj(R[i][c]).
 template <class T, int Q, int C, bool TRANS, class X>
-__device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* A, int lda, T* V, int ldv, T* tau,
+__device__ __noinline__ void qr_pass(const X ex, int m, int n, const T* A, int lda, T* V, T* Vwork, int ldv, T* tau,
                                      T* Rt, int ldr, T* vb) {
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
@@ -186,6 +186,9 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
   constexpr bool SKIP = sizeof(T) > 4;
   const int w4 = ex.warp() << 2;  // the warp's first group
   T* tb = vb + 2 * ldb;
+  if (!V && n > C * ngrp) V = Vwork;
+#pragma unroll 1
+  for (int c0 = 0; c0 < n; c0 += C * ngrp) {
   T x[C][Q * E];
 #pragma unroll
   for (int s = 0; s < C; ++s) {
@@ -279,20 +282,22 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, int c0, const T* 
     }
   }
   ex.sync();
+  }
 }
 
-// One register pass of Y = H_0 H_1 .. H_{k-1} [L; 0]: columns c0 .. of L (k x
+// Y = H_0 H_1 .. H_{k-1} [L; 0] in register passes over the columns of L (k x
 // nc, column-major; the identity when L is null).  Columns are independent,
 // so there is no barrier; v comes straight from V (cached).  Row i p + u of
 // column c goes to Y[(u nc + c) ldy + i] (p = pout): the columns of Y viewed
 // as cur x (pout nc).
 template <class T, int Q, int C, class X>
 __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, int ldv, const T* tau, const T* L,
-                                          int ldl, int nc, int c0, int pout, T* Y, int ldy) {
+                                          int ldl, int nc, int pout, T* Y, int ldy) {
   constexpr int E = Chunk<T>::E;
   const int li = ex.tid() & 7, grp = ex.tid() >> 3, ngrp = ex.size() >> 3;
   const int mp = (m + E - 1) / E * E, w4 = ex.warp() << 2;
-  if (c0 + w4 >= nc) return;  // no column for this warp
+#pragma unroll 1
+  for (int c0 = 0; c0 + w4 < nc; c0 += C * ngrp) {  // while there is a column for this warp
   T x[C][Q * E];
 #pragma unroll
   for (int s = 0; s < C; ++s) {
@@ -368,6 +373,8 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
         }
       }
   }
+  }
+  ex.sync();
 }
 
 // qr_factor for columns longer than the register variants take: the same
@@ -443,7 +450,11 @@ constexpr int jacobi_max_rows() { return sizeof(T) == 4 ? 256 : sizeof(T) == 8 ?
 
 // Register variants: chunks per lane Q (rows up to Q ROWS) and columns per
 // group C.  C is what keeps x within about 64 registers a thread (128 are
-// available) and, at the bench's sizes, takes every column in one pass.
+// available).  The dispatchers hold nothing after the call: a variant takes
+// nearly all registers, so whatever a caller keeps across it goes to local
+// memory and, with shared memory taking most of L1, on to L2 (this and AbsorbArgs:
+// 1824 chains of three boson lattices, four per CTA 4.79 -> 4.44 s; log-derivatives
+// 10x10, D_k = 3, chi = 36 91.2 -> 84.4 ms).
 #define GCF_QC_CASES(T, CALL)                                                        \
   if constexpr (sizeof(T) == 4) {                                                    \
     if (nq <= 1) { CALL(1, 3) } else if (nq <= 2) { CALL(2, 3) }                     \
@@ -467,12 +478,7 @@ template <class T, bool TRANS, class X>
 __device__ __noinline__ void qr_factor(const X ex, int m, int n, const T* A, int lda, T* V, T* Vwork, int ldv, T* tau, T* Rt,
                                        int ldr, T* vb) {
   const int nq = (m + Chunk<T>::ROWS - 1) / Chunk<T>::ROWS;
-  const int ngrp = ex.size() >> 3;
-#define GCF_QR_CALL(Qv, Cv)                                                                              \
-  T* v = V ? V : (n > Cv * ngrp ? Vwork : nullptr);                                                      \
-  for (int c0 = 0; c0 < n; c0 += Cv * ngrp)                                                              \
-    qr_pass<T, Qv, Cv, TRANS>(ex, m, n, c0, A, lda, v, ldv, tau, Rt, ldr, vb);                           \
-  return;
+#define GCF_QR_CALL(Qv, Cv) return qr_pass<T, Qv, Cv, TRANS>(ex, m, n, A, lda, V, Vwork, ldv, tau, Rt, ldr, vb);
   GCF_QC_CASES(T, GCF_QR_CALL)
 #undef GCF_QR_CALL
   qr_general<T, TRANS>(ex, m, n, A, lda, V != nullptr, V ? V : Vwork, ldv, tau, Rt, ldr);
@@ -486,14 +492,8 @@ __device__ __noinline__ void apply_q(const X ex, int m, int k, const T* V, int l
   const int nq = (m + Chunk<T>::ROWS - 1) / Chunk<T>::ROWS;
   const int ngrp = ex.size() >> 3;
 #define GCF_AQ_CALL(Qv, Cv)                                                                              \
-  if (nc <= ngrp) {                                                                                      \
-    apply_q_pass<T, Qv, 1>(ex, m, k, V, ldv, tau, L, ldl, nc, 0, pout, Y, ldy);                          \
-  } else {                                                                                               \
-    for (int c0 = 0; c0 < nc; c0 += Cv * ngrp)                                                           \
-      apply_q_pass<T, Qv, Cv>(ex, m, k, V, ldv, tau, L, ldl, nc, c0, pout, Y, ldy);                      \
-  }                                                                                                      \
-  ex.sync();                                                                                             \
-  return;
+  if (nc <= ngrp) return apply_q_pass<T, Qv, 1>(ex, m, k, V, ldv, tau, L, ldl, nc, pout, Y, ldy);        \
+  return apply_q_pass<T, Qv, Cv>(ex, m, k, V, ldv, tau, L, ldl, nc, pout, Y, ldy);
   GCF_QC_CASES(T, GCF_AQ_CALL)
 #undef GCF_AQ_CALL
   apply_q_general(ex, m, k, V, ldv, tau, L, ldl, nc, pout, Y, ldy, work, ldv);
@@ -607,10 +607,10 @@ __device__ __forceinline__ void apply_rot(T* a, T* b, typename Traits<T>::R c, T
 // the 12 pairs inside the blocks) are rotated, four disjoint pairs at a time.
 // Each quarter of the lanes forms the rotation of one pair (quarter i that of a_i); the squared norms
 // are summed once per meeting and moved along by the rotations, so a step
-// reduces only the four inner products.  Returns the sweeps used.
+// reduces only the four inner products.  Returns the sweeps used (max_sweeps: not
+// converged).
 template <class T, int LG, int R, class X>
-__device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int ldw, int* sflag, int max_sweeps,
-                                          int* converged) {
+__device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int ldw, int* sflag, int max_sweeps) {
   using S = typename Traits<T>::R;
   const int nb = kp >> 2, npair = nb >> 1;
   const int slots = ex.size() / LG, sub = ex.tid() / LG, li = ex.tid() & (LG - 1);
@@ -626,7 +626,6 @@ __device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int l
   f2 = ex.template sum<S>(f2);
   const S negl = Traits<T>::eps() * Traits<T>::eps() * f2;
   int sweep = 0;
-  *converged = 1;
   for (; sweep < max_sweeps; ++sweep) {
     if (ex.tid() == 0) *sflag = 0;
     ex.sync();
@@ -730,32 +729,30 @@ __device__ __noinline__ int jacobi_blocks(const X ex, int p, int kp, T* W, int l
     ex.sync();
     if (!any) break;
   }
-  if (sweep >= max_sweeps) *converged = 0;
   return sweep;
 }
 
 // Lanes per block pair and rows a lane by the column length p: 16 lanes while
 // 8 columns fit about 64 registers, else a warp.
 template <class T, class X>
-__device__ __noinline__ int jacobi_columns(const X ex, int p, int kp, T* W, int ldw, int* sflag, int max_sweeps,
-                                           int* converged) {
+__device__ __noinline__ int jacobi_columns(const X ex, int p, int kp, T* W, int ldw, int* sflag, int max_sweeps) {
   if constexpr (sizeof(T) == 4) {
-    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 32) return jacobi_blocks<T, 16, 2>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 48) return jacobi_blocks<T, 16, 3>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 80) return jacobi_blocks<T, 16, 5>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 128) return jacobi_blocks<T, 32, 4>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 256) return jacobi_blocks<T, 32, 8>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
+    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 32) return jacobi_blocks<T, 16, 2>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 48) return jacobi_blocks<T, 16, 3>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 80) return jacobi_blocks<T, 16, 5>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 128) return jacobi_blocks<T, 32, 4>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 256) return jacobi_blocks<T, 32, 8>(ex, p, kp, W, ldw, sflag, max_sweeps);
   } else if constexpr (sizeof(T) == 8) {
-    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 32) return jacobi_blocks<T, 16, 2>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 64) return jacobi_blocks<T, 32, 2>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 128) return jacobi_blocks<T, 32, 4>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
+    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 32) return jacobi_blocks<T, 16, 2>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 64) return jacobi_blocks<T, 32, 2>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 128) return jacobi_blocks<T, 32, 4>(ex, p, kp, W, ldw, sflag, max_sweeps);
   } else {
-    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
-    if (p <= 64) return jacobi_blocks<T, 32, 2>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
+    if (p <= 16) return jacobi_blocks<T, 16, 1>(ex, p, kp, W, ldw, sflag, max_sweeps);
+    if (p <= 64) return jacobi_blocks<T, 32, 2>(ex, p, kp, W, ldw, sflag, max_sweeps);
   }
-  return cta_jacobi<T>(ex, p, kp, W, ldw, sflag, max_sweeps, converged);
+  return cta_jacobi<T>(ex, p, kp, W, ldw, sflag, max_sweeps);
 }
 
 // G (kk x kk, column-major) <- (3 I - V^H V) / 2 for V (p x kk, column-major).

@@ -276,15 +276,14 @@ __shared__ long long g_fz_elems;  // scalars of each workspace
 
 // One-sided Jacobi on the columns of W (p x q, column-major), any size: on
 // return the columns are mutually orthogonal.  Returns the number of sweeps
-// used; *converged set to 0 if the sweep limit was hit.
+// used (max_sweeps: not converged).
 // Each sweep visits every column pair once in the round-robin order (n - 1
 // rounds of n/2 disjoint pairs, n = q rounded up to even).  A pair is served
 // by L consecutive lanes (the largest power of two <= 32 with L x n/2 within
 // the executor), which split its rows and combine their partial sums by
 // shuffles, so that all pairs of a round proceed at once.
 template <class T, class X>
-__device__ __noinline__ int cta_jacobi(const X ex, int p, int q, T* W, int ldw, int* sflag, int max_sweeps,
-                                       int* converged) {
+__device__ __noinline__ int cta_jacobi(const X ex, int p, int q, T* W, int ldw, int* sflag, int max_sweeps) {
   using R = typename Traits<T>::R;
   const int n = q + (q & 1);
   const int npair = n / 2;
@@ -308,7 +307,6 @@ __device__ __noinline__ int cta_jacobi(const X ex, int p, int q, T* W, int ldw, 
   f2 = ex.template sum<R>(f2);
   const R negl = Traits<T>::eps() * Traits<T>::eps() * f2;
   int sweep = 0;
-  if (converged) *converged = 1;
   for (; sweep < max_sweeps; ++sweep) {
     if (ex.tid() == 0) *sflag = 0;
     ex.sync();
@@ -378,7 +376,6 @@ __device__ __noinline__ int cta_jacobi(const X ex, int p, int q, T* W, int ldw, 
     ex.sync();
     if (!any) break;
   }
-  if (sweep >= max_sweeps && converged) *converged = 0;
   ex.sync();
   return sweep;
 }

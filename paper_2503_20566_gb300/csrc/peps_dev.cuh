@@ -108,7 +108,20 @@ struct KParams {
 enum { WANT_AMP = 1, WANT_ELOC = 2, WANT_GRAD = 4 };
 enum { ST_GAUSS = 0, ST_TC_TIMEOUT = 1, ST_SVD = 2, ST_PHASE_TIMEOUT = 3 };
 
+// What an absorption keeps across its factorisations, in shared memory: the
+// same for every thread of the chain, and those routines leave no registers for
+// it (one copy here instead of one per thread in local memory, i.e. L2).
+struct AbsorbArgs {
+  void *M1, *M2, *M3, *tau, *Qs, *Z, *Xb, *W1, *Vw, *W4, *sigma, *sel, *mout;
+  const void *net, *mps_in;
+  const int *bdi, *bdo, *qr, *svd;
+  int Lx, Dk, pin, pout, row, sd, su, max_sweeps;
+  int* status;  // KParams::status
+  void *w, *vs, *gg;  // truncate_bond
+};
+
 struct Shared {
+  AbsorbArgs ab_args;
   double red[64];
   double bcast;
   int iflag[4];
@@ -409,62 +422,74 @@ __device__ __noinline__ void site_product(const X ex, const SiteDims d, const T*
 // add the same squares in another order, and a column that they left alone may
 // lie along a leading one, so none of those may be kept.
 // Work: W, V and the Gram matrix in the chain's shared-memory workspace as
-// far as they fit it, else in g0, g1, g2 (mat_max each); Vwork, tau for the QR.
+// far as they fit it, else in M1, M2, M3 (mat_max each); Vw, tau for the QR.
+// Returns whether the sweeps converged.
 template <class T, class X>
-__device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, const T* Y, int ldy, T* carry, int ldl,
-                                           T* site, T* g0, T* g1, T* g2, T* Vwork, T* tau,
-                                           typename Traits<T>::R* sigma, int* sel, int* sflag, int max_sweeps,
-                                           int* conv) {
+__device__ __noinline__ bool truncate_bond(const X ex, Shared& sh, int yr, int yc, int kk, const T* Y, int ldy, T* carry,
+                                           int ldl, T* site) {
   using R = typename Traits<T>::R;
+  AbsorbArgs& g = sh.ab_args;
   const int k0 = min(yr, yc), kp = (k0 + 7) & ~7, ldw = pad4(yc);
-  const int nvb = qr_vb_elems<T>(yr), nw = ldw * kp, nv = ldw * kk, ng = pad4(kk * kk);
-  T* fz = (T*)g_fz[ex.slot()];
-  long long room = fz ? g_fz_elems : 0;
-  auto place = [&](long long n, T* other) {
-    if (n > room) return other;
-    T* q = fz;
-    fz += n;
-    room -= n;
-    return q;
-  };
-  T* vb = place(nvb, carry);  // the carry is written last
-  T* w = place(nw, g0);
-  T* vs = place(nv, g1);
-  T* gg = place(ng, g2);
+  {
+    const int nvb = qr_vb_elems<T>(yr), nw = ldw * kp, nv = ldw * kk, ng = pad4(kk * kk);
+    T* fz = (T*)g_fz[ex.slot()];
+    long long room = fz ? g_fz_elems : 0;
+    auto place = [&](long long n, void* other) {
+      if (n > room) return (T*)other;
+      T* q = fz;
+      fz += n;
+      room -= n;
+      return q;
+    };
+    T* vb = place(nvb, carry);  // the carry is written last
+    T* w = place(nw, g.M1);
+    T* vs = place(nv, g.M2);
+    T* gg = place(ng, g.M3);
+    if (ex.tid() == 0) { g.w = w; g.vs = vs; g.gg = gg; }
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < (kp - k0) * ldw; idx += ex.size()) w[k0 * ldw + idx] = zero<T>();
-  qr_factor<T, true>(ex, yr, yc, Y, ldy, (T*)nullptr, Vwork, ldy, tau, w, ldw, vb);
-  jacobi_columns<T>(ex, yc, kp, w, ldw, sflag, max_sweeps, conv);
-#pragma unroll 1
-  for (int j = ex.warp(); j < k0; j += ex.nwarps()) {
-    R s2 = R(0);
-    for (int i = ex.lane(); i < yc; i += 32) s2 += abs2(w[j * ldw + i]);
-    s2 = warp_sum(s2);
-    if (ex.lane() == 0) sigma[j] = s2;
+    for (int idx = ex.tid(); idx < (kp - k0) * ldw; idx += ex.size()) w[k0 * ldw + idx] = zero<T>();
+    qr_factor<T, true>(ex, yr, yc, Y, ldy, (T*)nullptr, (T*)g.Vw, ldy, (T*)g.tau, w, ldw, vb);
   }
-  ex.sync();
-  R f2 = R(0);
-  for (int j = ex.lane(); j < k0; j += 32) f2 += sigma[j];
-  f2 = warp_sum(f2);
-  const R negl = Traits<T>::eps() * Traits<T>::eps() * f2 * R(1 + 1.0 / 1024);
-  select_largest(ex, k0, kk, sigma, sel);
+  const bool conv = jacobi_columns<T>(ex, yc, kp, (T*)g.w, ldw, &sh.iflag[0], g.max_sweeps) < g.max_sweeps;
+  {
+    const T* w = (const T*)g.w;
+    T* vs = (T*)g.vs;
+    R* sigma = (R*)g.sigma;
+    int* sel = (int*)g.sel;
 #pragma unroll 1
-  for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
-    const int n = idx / yc, i = idx - (idx / yc) * yc;
-    const R s2 = sigma[sel[n]];
-    vs[n * ldw + i] = s2 > negl ? scale(w[sel[n] * ldw + i], R(1) / sqrt(s2)) : zero<T>();
+    for (int j = ex.warp(); j < k0; j += ex.nwarps()) {
+      R s2 = R(0);
+      for (int i = ex.lane(); i < yc; i += 32) s2 += abs2(w[j * ldw + i]);
+      s2 = warp_sum(s2);
+      if (ex.lane() == 0) sigma[j] = s2;
+    }
+    ex.sync();
+    R f2 = R(0);
+    for (int j = ex.lane(); j < k0; j += 32) f2 += sigma[j];
+    f2 = warp_sum(f2);
+    const R negl = Traits<T>::eps() * Traits<T>::eps() * f2 * R(1 + 1.0 / 1024);
+    select_largest(ex, k0, kk, sigma, sel);
+#pragma unroll 1
+    for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
+      const int n = idx / yc, i = idx - (idx / yc) * yc;
+      const R s2 = sigma[sel[n]];
+      vs[n * ldw + i] = s2 > negl ? scale(w[sel[n] * ldw + i], R(1) / sqrt(s2)) : zero<T>();
+    }
+    ex.sync();
   }
-  ex.sync();
-  gram_3i<T>(ex, yc, kk, vs, ldw, gg);
+  gram_3i<T>(ex, yc, kk, (const T*)g.vs, ldw, (T*)g.gg);
   // V' over W, which is not needed any more
-  cta_gemm_out<T>(ex, yc, kk, kk, vs, {1, 1, 0}, ldw, gg, 1, kk, OutMap<T>{w, {1, 1, 0}, kk, 0, ldw});
-  cta_gemm_out<T>(ex, yr, kk, yc, Y, {1, 1, 0}, ldy, w, 1, ldw, OutMap<T>{carry, {1, 1, 0}, kk, 0, ldl});
+  cta_gemm_out<T>(ex, yc, kk, kk, (const T*)g.vs, {1, 1, 0}, ldw, (const T*)g.gg, 1, kk,
+                  OutMap<T>{(T*)g.w, {1, 1, 0}, kk, 0, ldw});
+  cta_gemm_out<T>(ex, yr, kk, yc, Y, {1, 1, 0}, ldy, (const T*)g.w, 1, ldw, OutMap<T>{carry, {1, 1, 0}, kk, 0, ldl});
+  const T* w = (const T*)g.w;
 #pragma unroll 1
   for (int idx = ex.tid(); idx < kk * yc; idx += ex.size()) {
     const int n = idx / yc, i = idx - (idx / yc) * yc;
     site[idx] = conjg(w[n * ldw + i]);
   }
   ex.sync();
+  return conv;
 }
 
 // ---------------------------------------------------------------------------
@@ -484,33 +509,10 @@ __device__ __noinline__ void truncate_bond(const X ex, int yr, int yc, int kk, c
 // carry of the right sweep (kc columns) instead of being formed.
 // ---------------------------------------------------------------------------
 template <class T, class X>
-__device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* ws, T* hot_base, Shared& sh, const T* net,
-                                  const T* mps_in, const int* bdi, int pin, int row, int flip, T* mout,
-                                  const int* bdo, int pout, const int* qr, const int* svd, const int* offi,
-                                  const int* offo, int dense) {
-  const int Lx = k.Lx, Dk = k.Dk;
-  const int D3 = Dk * Dk * Dk, D2 = Dk * Dk;
-  const int sd = flip ? 1 : Dk, su = flip ? Dk : 1;
-  T* M1 = ws + k.o_M1;
-  T* M2 = ws + k.o_M2;
-  T* M3 = ws + k.o_M3;
-  T* tau = ws + k.o_tau;
-  T* Qs = ws + k.o_Q;
+__device__ __noinline__ int absorb_general(const X ex, Shared& sh) {
+  const AbsorbArgs& g = sh.ab_args;
+  const int Lx = g.Lx;
   int logs = 0;
-#pragma unroll 1
-  for (int c = ex.tid(); c <= Lx; c += ex.size()) {
-    sh.bd_off[c] = offi[c];
-    sh.bd_off2[c] = offo[c];
-  }
-  ex.sync();
-  // Dense (identity + core) path: every output bond at full rank and the
-  // dense state small enough (flag planned on the host).
-  if (dense) {
-    T* bufA = k.hot_in_smem ? hot_base + k.so_t1 : ws + k.o_t1;
-    T* bufB = k.hot_in_smem ? hot_base + k.so_t2 : ws + k.o_t2;
-    return dense_absorb<T>(ex, k, sh, net, mps_in, bdi, pin, row, flip, mout, bdo, pout, bufA, bufB);
-  }
-
   // General path.  Z_c (absorbed sites) right of cL; then a QR sweep from the
   // left over the bonds that must shrink (all bonds if the step truncates),
   // then a sweep from the right over the bonds that must shrink (truncated SVD,
@@ -524,6 +526,8 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   // 4x4, D_k = 3, chi = 9, complex FP32: 166 -> 156 us; 608 FP32 chains of 4x4
   // with bosons, four sweeps: 6.13 -> 5.80 ms).
   if (ex.tid() == 0) {
+    const int *bdi = g.bdi, *qr = g.qr, *svd = g.svd;
+    const int Dk = g.Dk, pout = g.pout;
     int any_svd = 0;
     for (int c = 1; c < Lx; ++c) any_svd |= svd[c];
     int zo = 0, qo = 0;
@@ -542,18 +546,14 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   }
   ex.sync();
   const int cL = sh.iflag[1];
-  T* Z = ws + k.o_Z;
-  T* Xb = ws + k.o_X;
-  T* Y = ws + k.o_W1;
-  T* Lc = ws + k.o_W4;
-  T* Vw = ws + k.o_W2;
   for (int c = cL ? cL + 1 : 0; c < Lx; ++c) {
-    const int a = bdi[c], b = bdi[c + 1];
+    const int Dk = g.Dk, pin = g.pin, pout = g.pout, sd = g.sd, su = g.su;
+    const int a = g.bdi[c], b = g.bdi[c + 1];
     const int l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
-    const T* M = mps_in + sh.bd_off[c];
-    const T* W = net + (long long)(row * Lx + c) * (Dk * Dk * Dk * Dk);
+    const T* M = (const T*)g.mps_in + sh.bd_off[c];
+    const T* W = (const T*)g.net + (long long)(g.row * Lx + c) * (Dk * Dk * Dk * Dk);
     const int nZ = a * l * pout * b * r;
-    T* Zc = Z + sh.zoff[c];
+    T* Zc = (T*)g.Z + sh.zoff[c];
 #pragma unroll 1
     for (int idx = ex.tid(); idx < nZ; idx += ex.size()) {
       int t = idx;
@@ -564,62 +564,69 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       const int ia = t;
       T s = zero<T>();
       for (int d = 0; d < pin; ++d)
-        s = fmac(s, M[(ia * pin + d) * b + ib], W[il * D3 + ir * D2 + d * sd + iu * su]);
+        s = fmac(s, M[(ia * pin + d) * b + ib], W[il * Dk * Dk * Dk + ir * Dk * Dk + d * sd + iu * su]);
       Zc[idx] = s;
     }
   }
   // ---- left QR sweep over sites 0..cL-1 (site cL: X only); carry Rc (Rrows x ab[c], column-major)
-  T* Rc = M3;
+  T* Rc = (T*)g.M3;
   if (ex.tid() == 0) Rc[0] = one<T>();
   ex.sync();
   int Rrows = 1, ldr = 4, ldxb = 4;
-  T* fz = (T*)g_fz[ex.slot()];
   for (int c = 0; c <= cL && cL; ++c) {
-    const int cols = sh.ab[c + 1], rows = Rrows * pout, ldx = pad4(rows);
-    const int nb = bdi[c + 1], l = hl_dim(c, Dk), r = hr_dim(c, Lx, Dk);
+    const int rows = Rrows * g.pout, ldx = pad4(rows);
     // X ((Rrows pout) x (b, r)) = sum R[.][(a l)] M[a][d][b] W[l][r][d][u], the
     // MPS site first: its a bond is the large one
-    T* Xc = (c == cL) ? Xb : (Rc == M3 ? M1 : M3);
-    T* T1 = M2;  // [(l d b)][Rrows]
-    const int ldt = pad4(Rrows);
-    cta_gemm_out<T>(ex, l * Rrows, pin * nb, bdi[c], Rc, {Rrows, ldr, 1}, l * ldr, mps_in + sh.bd_off[c], pin * nb, 1,
-                    OutMap<T>{T1, {Rrows, pin * nb * ldt, 1}, pin * nb, 0, ldt});
-    const T* W = net + (long long)(row * Lx + c) * (Dk * Dk * Dk * Dk);
-    const SiteDims sd_{l, r, pin, pout, sd, su, Rrows, nb, ldt, ldx};
-    switch (Dk) {
-      case 1: site_product<T, 1>(ex, sd_, W, T1, Xc); break;
-      case 2: site_product<T, 2>(ex, sd_, W, T1, Xc); break;
-      default: site_product<T, 3>(ex, sd_, W, T1, Xc); break;
+    T* Xc = (T*)(c == cL ? g.Xb : Rc == g.M3 ? g.M1 : g.M3);
+    {
+      const int nb = g.bdi[c + 1], pin = g.pin, Dk = g.Dk, l = hl_dim(c, Dk), ldt = pad4(Rrows);
+      T* T1 = (T*)g.M2;  // [(l d b)][Rrows]
+      cta_gemm_out<T>(ex, l * Rrows, pin * nb, g.bdi[c], Rc, {Rrows, ldr, 1}, l * ldr, (const T*)g.mps_in + sh.bd_off[c],
+                      pin * nb, 1, OutMap<T>{T1, {Rrows, pin * nb * ldt, 1}, pin * nb, 0, ldt});
+    }
+    {
+      const int Dk = g.Dk;
+      const T* W = (const T*)g.net + (long long)(g.row * Lx + c) * (Dk * Dk * Dk * Dk);
+      const SiteDims d{hl_dim(c, Dk), hr_dim(c, Lx, Dk), g.pin, g.pout, g.sd, g.su, Rrows, g.bdi[c + 1], pad4(Rrows), ldx};
+      switch (Dk) {
+        case 1: site_product<T, 1>(ex, d, W, (const T*)g.M2, Xc); break;
+        case 2: site_product<T, 2>(ex, d, W, (const T*)g.M2, Xc); break;
+        default: site_product<T, 3>(ex, d, W, (const T*)g.M2, Xc); break;
+      }
     }
     ldxb = ldx;
     if (c == cL) break;
+    const int cols = sh.ab[c + 1];
     if (rows <= cols) {
       Rc = Xc;
       ldr = ldx;
       Rrows = rows;
     } else {
-      T* V = Qs + sh.qoff[c];
-      T* vb = (fz && qr_vb_elems<T>(rows) <= g_fz_elems) ? fz : M2;
+      T* V = (T*)g.Qs + sh.qoff[c];
+      T* fz = (T*)g_fz[ex.slot()];
       ldr = pad4(cols);
-      qr_factor<T, false>(ex, rows, cols, Xc, ldx, V, (T*)nullptr, ldx, V + ldx * cols, Rc, ldr, vb);
+      qr_factor<T, false>(ex, rows, cols, Xc, ldx, V, (T*)nullptr, ldx, V + ldx * cols, Rc, ldr,
+                          (fz && qr_vb_elems<T>(rows) <= g_fz_elems) ? fz : (T*)g.M2);
       Rrows = cols;
     }
-    logs += frob_rescale_cm(ex, Rrows, cols, Rc, ldr);
+    logs += frob_rescale_cm(ex, Rrows, sh.ab[c + 1], Rc, ldr);
   }
   // ---- right sweep over every site.  The carry Lc (rd x kc, column-major) is
   // the identity while no bond to the right has been reduced.
   // Y (cur x (pout, kc), column-major): site c times the carry.
   bool ident = true;
   int kc = 1, ldl = 4;
+  T* Y = (T*)g.W1;
+  T* Lc = (T*)g.W4;
   for (int c = Lx - 1; c >= 0; --c) {
-    const int cur = (c < cL) ? qr[c] : (c == cL ? Rrows : sh.ab[c]);
-    const int rd = (c < cL) ? qr[c + 1] : sh.ab[c + 1];
-    const int n = ident ? rd : kc, yc = pout * n, ldy = pad4(cur), rows = cur * pout;
-    const bool from_x = c == cL && cL, shrinks = c >= 1 && (svd[c] || bdo[c] < cur);
-    const T* S = from_x ? Xb : Z + sh.zoff[c];
-    T* site = mout + sh.bd_off2[c];
+    const int cur = (c < cL) ? g.qr[c] : (c == cL ? Rrows : sh.ab[c]);
+    const int rd = (c < cL) ? g.qr[c + 1] : sh.ab[c + 1];
+    const int pout = g.pout, n = ident ? rd : kc, yc = pout * n, ldy = pad4(cur), rows = cur * pout;
+    const bool from_x = c == cL && cL, shrinks = c >= 1 && (g.svd[c] || g.bdo[c] < cur);
+    T* site = (T*)g.mout + sh.bd_off2[c];
     if (ident && c >= cL && !shrinks) {
       // the absorbed site as it is
+      const T* S = from_x ? (const T*)g.Xb : (const T*)g.Z + sh.zoff[c];
 #pragma unroll 1
       for (int idx = ex.tid(); idx < rows * n; idx += ex.size())
         site[idx] = from_x ? S[(idx % n) * ldxb + idx / n] : S[idx];
@@ -628,11 +635,12 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       continue;
     }
     if (c < cL && rows > rd) {
-      const T* V = Qs + sh.qoff[c];
+      const T* V = (const T*)g.Qs + sh.qoff[c];
       const int ldv = pad4(rows);
-      apply_q<T>(ex, rows, rd, V, ldv, V + ldv * rd, ident ? (const T*)nullptr : Lc, ldl, n, pout, Y, ldy, M1);
+      apply_q<T>(ex, rows, rd, V, ldv, V + ldv * rd, ident ? (const T*)nullptr : Lc, ldl, n, pout, Y, ldy, (T*)g.M1);
     } else if (c < cL || ident) {
       // identity isometry (Y = the carry) or identity carry (Y = the site)
+      const T* S = from_x ? (const T*)g.Xb : (const T*)g.Z + sh.zoff[c];
 #pragma unroll 1
       for (int idx = ex.tid(); idx < rows * n; idx += ex.size()) {
         const int m = idx / rows, q = idx - (idx / rows) * rows;
@@ -644,12 +652,13 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
       }
       ex.sync();
     } else {
+      const T* S = from_x ? (const T*)g.Xb : (const T*)g.Z + sh.zoff[c];
       cta_gemm_out<T>(ex, rows, n, rd, S, {1, from_x ? 1 : rd, 0}, from_x ? ldxb : 1, Lc, 1, ldl,
                       OutMap<T>{Y, {pout, 1, n * ldy}, n, 0, ldy});
     }
     if (shrinks) {
-      const int kk = bdo[c];
-      if (!svd[c]) {
+      const int kk = g.bdo[c];
+      if (!g.svd[c]) {
         // yc = kk columns already fit the bond: the identity is the isometry
 #pragma unroll 1
         for (int idx = ex.tid(); idx < kk * yc; idx += ex.size())
@@ -657,15 +666,12 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
         T* t = Lc; Lc = Y; Y = t;
         ldl = ldy;
       } else {
-        using RR = typename Traits<T>::R;
-        int conv = 1;
         ldl = pad4(cur);
-        truncate_bond<T>(ex, cur, yc, kk, Y, ldy, Lc, ldl, site, M1, M2, M3, Vw, tau, (RR*)(ws + k.o_sigma),
-                         (int*)(ws + k.o_sel), &sh.iflag[0], k.max_sweeps_svd, &conv);
-        if (!conv && ex.tid() == 0) atomicAdd(&k.status[ST_SVD], 1);
+        if (!truncate_bond<T>(ex, sh, cur, yc, kk, Y, ldy, Lc, ldl, site) && ex.tid() == 0)
+          atomicAdd(&g.status[ST_SVD], 1);
       }
-      logs += frob_rescale_cm(ex, cur, kk, Lc, ldl);
-      kc = kk;
+      logs += frob_rescale_cm(ex, cur, g.bdo[c], Lc, ldl);
+      kc = g.bdo[c];
       ident = false;
     } else {
       // no reduction at this site's left bond (cur == bdo[c]): keep Y
@@ -682,4 +688,33 @@ __device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* 
   return logs;
 }
 
+template <class T, class X>
+__device__ __noinline__ int absorb_compress(const X ex, const KParams<T>& k, T* ws, T* hot_base, Shared& sh, const T* net,
+                                  const T* mps_in, const int* bdi, int pin, int row, int flip, T* mout,
+                                  const int* bdo, int pout, const int* qr, const int* svd, const int* offi,
+                                  const int* offo, int dense) {
+#pragma unroll 1
+  for (int c = ex.tid(); c <= k.Lx; c += ex.size()) {
+    sh.bd_off[c] = offi[c];
+    sh.bd_off2[c] = offo[c];
+  }
+  ex.sync();
+  // Dense (identity + core) path: every output bond at full rank and the
+  // dense state small enough (flag planned on the host).
+  if (dense) {
+    T* bufA = k.hot_in_smem ? hot_base + k.so_t1 : ws + k.o_t1;
+    T* bufB = k.hot_in_smem ? hot_base + k.so_t2 : ws + k.o_t2;
+    return dense_absorb<T>(ex, k, sh, net, mps_in, bdi, pin, row, flip, mout, bdo, pout, bufA, bufB);
+  }
+  if (ex.tid() == 0) {
+    AbsorbArgs& a = sh.ab_args;
+    a.M1 = ws + k.o_M1; a.M2 = ws + k.o_M2; a.M3 = ws + k.o_M3; a.tau = ws + k.o_tau; a.Qs = ws + k.o_Q;
+    a.Z = ws + k.o_Z; a.Xb = ws + k.o_X; a.W1 = ws + k.o_W1; a.Vw = ws + k.o_W2; a.W4 = ws + k.o_W4; a.sigma = ws + k.o_sigma; a.sel = ws + k.o_sel;
+    a.mout = mout; a.net = net; a.mps_in = mps_in; a.bdi = bdi; a.bdo = bdo; a.qr = qr; a.svd = svd;
+    a.Lx = k.Lx; a.Dk = k.Dk; a.pin = pin; a.pout = pout; a.row = row;
+    a.sd = flip ? 1 : k.Dk; a.su = flip ? k.Dk : 1; a.max_sweeps = k.max_sweeps_svd; a.status = k.status;
+  }
+  ex.sync();
+  return absorb_general<T>(ex, sh);
+}
 }  // namespace gcf
