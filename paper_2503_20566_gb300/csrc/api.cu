@@ -879,12 +879,14 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     ks[i].fz_elems = fz;
     ks[i].fz_off = (long long)fz_off;
   }
-  // One chain per CTA (vmc_kernel_multi) where two CTAs fit an SM: 338 samples/s
-  // on the 16x16 + 24x24 + 32x32 boson mix (chi = 24) against 326 with four
-  // chains per CTA (vmc_kernel_multi4, hot buffers in scratch), and fewer
-  // chains spread over more SMs.  Truncating contexts whose shared memory or
-  // tcgen05 instructions leave one CTA per SM take four chains per CTA.
-  // GCFVMC_MULTI=cta|group4 forces a form.
+  // Truncating contexts take four chains per CTA (vmc_kernel_multi4, hot buffers
+  // in scratch) from three rounds of one chain per CTA (vmc_kernel_multi) on:
+  // the factorisations wait on their own steps, and more chains per SM fill the
+  // waits once all SMs are busy anyway; below, a chain on a whole CTA ends
+  // sooner.  16x16 + 24x24 + 32x32 bosons, chi = 24 (one per CTA, four per CTA):
+  // FP32 (two CTAs per SM) 1824 chains 4.89 s, 4.43 s; 1026: 2.93, 2.68; 609: 1.95,
+  // 2.40; 60: 1.27, 1.83; BF16 (tcgen05: one CTA per SM) 1026: 4.96, 3.05; 303:
+  // 1.53, 2.29.  GCFVMC_MULTI=cta|group4 forces a form.
   int block = 256;
   long long group_bytes = 0;
   {
@@ -893,7 +895,8 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     const size_t g_tc = (sharedv_bytes() + cfg_max + 15) / 16 * 16;
     const size_t g_fz = g_tc;
     const size_t gb = (g_tc + area + 15) / 16 * 16;
-    bool want4 = fz > 0 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi, smem) < 2;
+    const int cta_slots = c0->sms * std::max(1, GCF_TC_CALL(T, tc_all, occupancy_vmc_multi, smem));
+    bool want4 = fz > 0 && total >= 3LL * cta_slots;
     if (const char* e = std::getenv("GCFVMC_MULTI")) want4 = !std::strcmp(e, "group4");
     if (want4 && 4 * gb <= 216 * 1024 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi4, 4 * gb) >= 1) {
       block = 512;
