@@ -12,8 +12,9 @@
 // Measured against the same steps with every column in shared memory or L2 (a
 // barrier and a pass over the matrix per column or column pair) and Q and J
 // formed: log-derivatives at 16x16, chi = 24, 304 configurations 117.7 -> 63.8
-// ms (43 with two blocks per SM); 10x10, D_k = 3, chi = 36, complex, 152
-// configurations 403 -> 159 ms (94 with 512 threads a chain).
+// ms (43 with two blocks per SM, 40 with IEEE divisions in the reflectors and
+// nothing held across a factorisation); 10x10, D_k = 3, chi = 36, complex, 152
+// configurations 403 -> 159 ms (94 with 512 threads a chain, 84 with those two).
 //
 // All matrices are column-major with leading dimensions padded to 4 rows
 // (pad4), so a lane moves 16 bytes of a column at a time.
@@ -189,99 +190,99 @@ __device__ __noinline__ void qr_pass(const X ex, int m, int n, const T* A, int l
   if (!V && n > C * ngrp) V = Vwork;
 #pragma unroll 1
   for (int c0 = 0; c0 < n; c0 += C * ngrp) {
-  T x[C][Q * E];
+    T x[C][Q * E];
 #pragma unroll
-  for (int s = 0; s < C; ++s) {
-    const int c = c0 + s * ngrp + grp;
+    for (int s = 0; s < C; ++s) {
+      const int c = c0 + s * ngrp + grp;
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int row = E * (li + 8 * q);
-      if (c < n && row < mp) {
-        load_chunk(x[s] + q * E, A + (long long)c * lda + row);
+      for (int q = 0; q < Q; ++q) {
+        const int row = E * (li + 8 * q);
+        if (c < n && row < mp) {
+          load_chunk(x[s] + q * E, A + (long long)c * lda + row);
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-          if (row + e >= m) x[s][q * E + e] = zero<T>();
-      } else {
+          for (int e = 0; e < E; ++e)
+            if (row + e >= m) x[s][q * E + e] = zero<T>();
+        } else {
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[s][q * E + e] = zero<T>();
-      }
-    }
-  }
-  for (int j = 0; j < min(c0, k); ++j) {
-    const T f = conjg(tau[j]);
-#pragma unroll
-    for (int s = 0; s < C; ++s)
-      if (c0 + s * ngrp + w4 < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
-  }
-  if (c0 < k && ex.warp() == 0)
-    make_reflector<T, Q>(x[0], c0, nq, li, grp == 0, vb + (c0 & 1) * ldb, tb + (c0 & 1));
-#pragma unroll
-  for (int s = 0; s < C; ++s) {
-#pragma unroll 1
-    for (int jj = 0; jj < ngrp; ++jj) {
-      const int j = c0 + s * ngrp + jj;
-      if (j >= k) break;
-      ex.sync();
-      const T* v = vb + (j & 1) * ldb;
-      const T f = conjg(tb[j & 1]);
-      const int q0 = j / (8 * E);
-      if (ex.tid() == 0 && V) tau[j] = tb[j & 1];
-      const bool cur = !SKIP || (w4 + 3 > jj && c0 + s * ngrp + w4 < n);  // columns of slot s left to this warp
-      if constexpr (C > 1) {
-        if (SKIP && !cur && !(s + 1 < C && c0 + (s + 1) * ngrp + w4 < n)) continue;
-        T vr[Q * E];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          if (q < nq) load_chunk(vr + q * E, v + E * (li + 8 * q));
-          else {
-#pragma unroll
-            for (int e = 0; e < E; ++e) vr[q * E + e] = zero<T>();
-          }
+          for (int e = 0; e < E; ++e) x[s][q * E + e] = zero<T>();
         }
-        if (cur) reflect_col<T, Q>(x[s], vr, grp > jj ? f : zero<T>(), q0);
-        if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
-          make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
-#pragma unroll
-        for (int s2 = s + 1; s2 < C; ++s2)
-          if (c0 + s2 * ngrp + (SKIP ? w4 : 0) < n) reflect_col<T, Q>(x[s2], vr, f, q0);
-      } else {
-        if (!cur) continue;
-        reflect_col_mem<T, Q>(x[s], v, li, grp > jj ? f : zero<T>(), q0, ldb);
-        if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
-          make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
-      }
-      if (s + 1 < C && jj == ngrp - 1 && ex.warp() == 0 && j + 1 < k)
-        make_reflector<T, Q>(x[s + 1 < C ? s + 1 : s], j + 1, nq, li, grp == 0, vb + ((j + 1) & 1) * ldb,
-                             tb + ((j + 1) & 1));
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < C; ++s) {
-    const int c = c0 + s * ngrp + grp;
-    if (c >= n) continue;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int row = E * (li + 8 * q);
-      if (TRANS) {
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          if (row + e < k) Rt[c + (long long)(row + e) * ldr] = row + e <= c ? conjg(x[s][q * E + e]) : zero<T>();
-      } else if (row < ldr) {
-        T o[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) o[e] = row + e <= c && row + e < k ? x[s][q * E + e] : zero<T>();
-        store_chunk(Rt + (long long)c * ldr + row, o);
-      }
-      if (V && c < k && row < mp) {
-        T o[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-          o[e] = row + e < c ? zero<T>() : row + e == c ? one<T>() : x[s][q * E + e];
-        store_chunk(V + (long long)c * ldv + row, o);
       }
     }
-  }
-  ex.sync();
+    for (int j = 0; j < min(c0, k); ++j) {
+      const T f = conjg(tau[j]);
+#pragma unroll
+      for (int s = 0; s < C; ++s)
+        if (c0 + s * ngrp + w4 < n) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
+    }
+    if (c0 < k && ex.warp() == 0)
+      make_reflector<T, Q>(x[0], c0, nq, li, grp == 0, vb + (c0 & 1) * ldb, tb + (c0 & 1));
+#pragma unroll
+    for (int s = 0; s < C; ++s) {
+#pragma unroll 1
+      for (int jj = 0; jj < ngrp; ++jj) {
+        const int j = c0 + s * ngrp + jj;
+        if (j >= k) break;
+        ex.sync();
+        const T* v = vb + (j & 1) * ldb;
+        const T f = conjg(tb[j & 1]);
+        const int q0 = j / (8 * E);
+        if (ex.tid() == 0 && V) tau[j] = tb[j & 1];
+        const bool cur = !SKIP || (w4 + 3 > jj && c0 + s * ngrp + w4 < n);  // columns of slot s left to this warp
+        if constexpr (C > 1) {
+          if (SKIP && !cur && !(s + 1 < C && c0 + (s + 1) * ngrp + w4 < n)) continue;
+          T vr[Q * E];
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            if (q < nq) load_chunk(vr + q * E, v + E * (li + 8 * q));
+            else {
+#pragma unroll
+              for (int e = 0; e < E; ++e) vr[q * E + e] = zero<T>();
+            }
+          }
+          if (cur) reflect_col<T, Q>(x[s], vr, grp > jj ? f : zero<T>(), q0);
+          if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
+            make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
+#pragma unroll
+          for (int s2 = s + 1; s2 < C; ++s2)
+            if (c0 + s2 * ngrp + (SKIP ? w4 : 0) < n) reflect_col<T, Q>(x[s2], vr, f, q0);
+        } else {
+          if (!cur) continue;
+          reflect_col_mem<T, Q>(x[s], v, li, grp > jj ? f : zero<T>(), q0, ldb);
+          if ((jj + 1) >> 2 == ex.warp() && jj + 1 < ngrp && j + 1 < k)
+            make_reflector<T, Q>(x[s], j + 1, nq, li, grp == jj + 1, vb + ((j + 1) & 1) * ldb, tb + ((j + 1) & 1));
+        }
+        if (s + 1 < C && jj == ngrp - 1 && ex.warp() == 0 && j + 1 < k)
+          make_reflector<T, Q>(x[s + 1 < C ? s + 1 : s], j + 1, nq, li, grp == 0, vb + ((j + 1) & 1) * ldb,
+                               tb + ((j + 1) & 1));
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < C; ++s) {
+      const int c = c0 + s * ngrp + grp;
+      if (c >= n) continue;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int row = E * (li + 8 * q);
+        if (TRANS) {
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            if (row + e < k) Rt[c + (long long)(row + e) * ldr] = row + e <= c ? conjg(x[s][q * E + e]) : zero<T>();
+        } else if (row < ldr) {
+          T o[E];
+#pragma unroll
+          for (int e = 0; e < E; ++e) o[e] = row + e <= c && row + e < k ? x[s][q * E + e] : zero<T>();
+          store_chunk(Rt + (long long)c * ldr + row, o);
+        }
+        if (V && c < k && row < mp) {
+          T o[E];
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            o[e] = row + e < c ? zero<T>() : row + e == c ? one<T>() : x[s][q * E + e];
+          store_chunk(V + (long long)c * ldv + row, o);
+        }
+      }
+    }
+    ex.sync();
   }
 }
 
@@ -298,81 +299,81 @@ __device__ __noinline__ void apply_q_pass(const X ex, int m, int k, const T* V, 
   const int mp = (m + E - 1) / E * E, w4 = ex.warp() << 2;
 #pragma unroll 1
   for (int c0 = 0; c0 + w4 < nc; c0 += C * ngrp) {  // while there is a column for this warp
-  T x[C][Q * E];
+    T x[C][Q * E];
 #pragma unroll
-  for (int s = 0; s < C; ++s) {
-    const int c = c0 + s * ngrp + grp;
+    for (int s = 0; s < C; ++s) {
+      const int c = c0 + s * ngrp + grp;
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
+      for (int q = 0; q < Q; ++q)
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int row = E * (li + 8 * q) + e;
-        x[s][q * E + e] = (c < nc && row < k) ? (L ? L[(long long)c * ldl + row] : (row == c ? one<T>() : zero<T>()))
-                                              : zero<T>();
-      }
-  }
-  // v of the next AHEAD steps are under way while one is applied (the reads
-  // come from L2), as far as registers allow; else v is read twice in place
-  constexpr int W = Q * E * (int)sizeof(T) / 4;  // registers of a column
-  constexpr int AHEAD = C * W >= 80 ? 0 : (80 - C * W) / W < 3 ? (80 - C * W) / W : 3;
-  auto fetch = [&](T* r, int j) {
-    const T* v = V + (long long)max(j, 0) * ldv;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int row = E * (li + 8 * q);
-      if (row < mp) load_chunk(r + q * E, v + row);
-      else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[q * E + e] = zero<T>();
-      }
+        for (int e = 0; e < E; ++e) {
+          const int row = E * (li + 8 * q) + e;
+          x[s][q * E + e] = (c < nc && row < k) ? (L ? L[(long long)c * ldl + row] : (row == c ? one<T>() : zero<T>()))
+                                                : zero<T>();
+        }
     }
-  };
-  if constexpr (AHEAD > 0) {
-    T vr[AHEAD][Q * E];
-    T fr[AHEAD];
+    // v of the next AHEAD steps are under way while one is applied (the reads
+    // come from L2), as far as registers allow; else v is read twice in place
+    constexpr int W = Q * E * (int)sizeof(T) / 4;  // registers of a column
+    constexpr int AHEAD = C * W >= 80 ? 0 : (80 - C * W) / W < 3 ? (80 - C * W) / W : 3;
+    auto fetch = [&](T* r, int j) {
+      const T* v = V + (long long)max(j, 0) * ldv;
 #pragma unroll
-    for (int a = 0; a < AHEAD; ++a) {
-      fetch(vr[a], k - 1 - a);
-      fr[a] = tau[max(k - 1 - a, 0)];
-    }
-#pragma unroll 1
-    for (int j0 = k - 1; j0 >= 0; j0 -= AHEAD) {
+      for (int q = 0; q < Q; ++q) {
+        const int row = E * (li + 8 * q);
+        if (row < mp) load_chunk(r + q * E, v + row);
+        else {
 #pragma unroll
-      for (int a = 0; a < AHEAD; ++a) {
-        const int j = j0 - a;
-        if (j < 0) break;
-        const int q0 = j / (8 * E);
-#pragma unroll
-        for (int s = 0; s < C; ++s)
-          if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0);
-        fetch(vr[a], j - AHEAD);
-        fr[a] = tau[max(j - AHEAD, 0)];
-      }
-    }
-  } else {
-#pragma unroll 1
-    for (int j = k - 1; j >= 0; --j) {
-      const T f = tau[j];
-#pragma unroll
-      for (int s = 0; s < C; ++s)
-        if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < C; ++s) {
-    const int c = c0 + s * ngrp + grp;
-    if (c >= nc) continue;
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int row = E * (li + 8 * q) + e;
-        if (row < m) {
-          const int i = row / pout, u = row - i * pout;
-          Y[(long long)(u * nc + c) * ldy + i] = x[s][q * E + e];
+          for (int e = 0; e < E; ++e) r[q * E + e] = zero<T>();
         }
       }
-  }
+    };
+    if constexpr (AHEAD > 0) {
+      T vr[AHEAD][Q * E];
+      T fr[AHEAD];
+#pragma unroll
+      for (int a = 0; a < AHEAD; ++a) {
+        fetch(vr[a], k - 1 - a);
+        fr[a] = tau[max(k - 1 - a, 0)];
+      }
+#pragma unroll 1
+      for (int j0 = k - 1; j0 >= 0; j0 -= AHEAD) {
+#pragma unroll
+        for (int a = 0; a < AHEAD; ++a) {
+          const int j = j0 - a;
+          if (j < 0) break;
+          const int q0 = j / (8 * E);
+#pragma unroll
+          for (int s = 0; s < C; ++s)
+            if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col<T, Q>(x[s], vr[a], fr[a], q0);
+          fetch(vr[a], j - AHEAD);
+          fr[a] = tau[max(j - AHEAD, 0)];
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int j = k - 1; j >= 0; --j) {
+        const T f = tau[j];
+#pragma unroll
+        for (int s = 0; s < C; ++s)
+          if (s == 0 || c0 + s * ngrp + w4 < nc) reflect_col_mem<T, Q>(x[s], V + (long long)j * ldv, li, f, j / (8 * E), mp);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < C; ++s) {
+      const int c = c0 + s * ngrp + grp;
+      if (c >= nc) continue;
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int row = E * (li + 8 * q) + e;
+          if (row < m) {
+            const int i = row / pout, u = row - i * pout;
+            Y[(long long)(u * nc + c) * ldy + i] = x[s][q * E + e];
+          }
+        }
+    }
   }
   ex.sync();
 }
@@ -537,6 +538,16 @@ __device__ __forceinline__ typename Traits<T>::R norm_col(const T* a) {
 // orthogonal: w_a <- c w_a - conj(se) w_b, w_b <- se w_a + c w_b with
 // se = s g / |g|.  Leaves c = 1, se = 0 (rot = false) when the pair is
 // orthogonal to rounding or a column is noise; moves the norms along.
+// In FP32 the angle comes from the hardware's reciprocal and square root: it
+// decides how fast the sweeps converge, not how orthogonal they leave the
+// columns (c^2 + s^2 = 1 to rounding for any angle, and the last sweep, which
+// rotates nothing, tests norms summed afresh).  With IEEE operations in their
+// place the errors against FP64 restatements are the same within their scatter
+// (two sets of inputs each, IEEE / hardware: amplitudes 32x32 3.0e-8 / 3.0e-8 and
+// 3.3e-8 / 3.4e-8; log-derivatives 16x16 1.6e-7 in all four, 10x10 complex 2.6e-7 /
+// 2.5e-7 and 2.3e-7 / 2.3e-7; E_loc 12x9 5.2e-7 / 5.1e-7 and 5.2e-7 / 5.2e-7, 16x16 Z3
+// 4.1e-7 / 5.9e-7 and 4.1e-6 / 2.0e-6), complex cases take 2 to 3 % longer and real
+// ones 1 % less.
 template <class T>
 __device__ __forceinline__ bool pair_rotation(typename Traits<T>::R& al, typename Traits<T>::R& be, T g,
                                               typename Traits<T>::R negl, typename Traits<T>::R tol,

@@ -603,7 +603,7 @@ __global__ void k_scatter_sorted(SrGeom g, const int* perm, const int* seg, int 
 // rows: 80 us at 1024 complex samples of 16x16 Z3).  Segments are split by their
 // own length: near a ground state one block of a vertex holds most samples (16000
 // complex samples of 8x8 Z4 with matter, nine in ten on one block, 20 CG steps:
-// 92 ms with a warp for a whole segment, 28 with a CTA, 5.7 in parts).  Warp w of
+// 93 ms with a warp for a whole segment, 28 with a CTA, 7.1 in parts).  Warp w of
 // vertex blockIdx.y finds its segment in the table of parts.
 template <class T, bool CONJ, bool CPLX, bool SQ>
 __global__ void k_scatter_warp(SrGeom g, const int* perm, const int* seg, const int* part_of, int maxnb, const T* osort,
