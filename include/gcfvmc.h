@@ -373,7 +373,7 @@ int gcf_tensor_timeouts(const gcf_ctx* ctx);
  * gcf::vmc_kernel_multi (one chain per CTA of 256 threads), 4 for
  * gcf::vmc_kernel_multi4 (four chains per CTA of 512 threads, chosen when a
  * context truncates and the chains are at least three times what the GPU holds
- * in the other form; GCFVMC_MULTI=cta|group4 forces one), 0 before any launch, -1 for a NULL
+ * in the other form, with the same results; GCFVMC_MULTI=cta|group4 forces one), 0 before any launch, -1 for a NULL
  * context. */
 int gcf_multi_chains_per_cta(const gcf_ctx* ctx);
 

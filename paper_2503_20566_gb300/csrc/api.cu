@@ -886,7 +886,8 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
   // sooner.  16x16 + 24x24 + 32x32 bosons, chi = 24 (one per CTA, four per CTA):
   // FP32 (two CTAs per SM) 1824 chains 4.89 s, 4.43 s; 1026: 2.93, 2.68; 609: 1.95,
   // 2.40; 60: 1.27, 1.83; BF16 (tcgen05: one CTA per SM) 1026: 4.96, 3.05; 303:
-  // 1.53, 2.29.  GCFVMC_MULTI=cta|group4 forces a form.
+  // 1.53, 2.29.  The chains are the same in both (see sum_size).
+  // GCFVMC_MULTI=cta|group4 forces a form.
   int block = 256;
   long long group_bytes = 0;
   {
@@ -896,7 +897,9 @@ gcf_status run_multi(gcf_ctx* const* cs, int n_ctx, const int* n_chains, int n_s
     const size_t g_fz = g_tc;
     const size_t gb = (g_tc + area + 15) / 16 * 16;
     const int cta_slots = c0->sms * std::max(1, GCF_TC_CALL(T, tc_all, occupancy_vmc_multi, smem));
-    bool want4 = fz > 0 && total >= 3LL * cta_slots;
+    bool general = false;  // results depend on the form: one form for any number of chains
+    for (int i = 0; i < n_ctx; ++i) general |= cs[i]->plan.general;
+    bool want4 = fz > 0 && (general ? cta_slots < 2 * c0->sms : total >= 3LL * cta_slots);
     if (const char* e = std::getenv("GCFVMC_MULTI")) want4 = !std::strcmp(e, "group4");
     if (want4 && 4 * gb <= 216 * 1024 && GCF_TC_CALL(T, tc_all, occupancy_vmc_multi4, 4 * gb) >= 1) {
       block = 512;

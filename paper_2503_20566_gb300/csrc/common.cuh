@@ -61,8 +61,11 @@ __host__ __device__ inline double im(cdouble a) { return a.y; }
 
 __host__ __device__ inline float abs2(float a) { return a * a; }
 __host__ __device__ inline double abs2(double a) { return a * a; }
-__host__ __device__ inline float abs2(cfloat a) { return a.x * a.x + a.y * a.y; }
-__host__ __device__ inline double abs2(cdouble a) { return a.x * a.x + a.y * a.y; }
+// Complex squares and products name their fused operations: left to the
+// compiler, the one that is fused can differ from kernel to kernel, and a chain's
+// last bits with it.
+__device__ inline float abs2(cfloat a) { return fmaf(a.x, a.x, __fmul_rn(a.y, a.y)); }
+__device__ inline double abs2(cdouble a) { return fma(a.x, a.x, __dmul_rn(a.y, a.y)); }
 
 __host__ __device__ inline float absmax1(float a) { return fabsf(a); }
 __host__ __device__ inline double absmax1(double a) { return fabs(a); }
@@ -75,11 +78,11 @@ __host__ __device__ inline cfloat operator-(cfloat a, cfloat b) { return {a.x - 
 __host__ __device__ inline cdouble operator-(cdouble a, cdouble b) { return {a.x - b.x, a.y - b.y}; }
 __host__ __device__ inline cfloat operator-(cfloat a) { return {-a.x, -a.y}; }
 __host__ __device__ inline cdouble operator-(cdouble a) { return {-a.x, -a.y}; }
-__host__ __device__ inline cfloat operator*(cfloat a, cfloat b) {
-  return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+__device__ inline cfloat operator*(cfloat a, cfloat b) {
+  return {fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x))};
 }
-__host__ __device__ inline cdouble operator*(cdouble a, cdouble b) {
-  return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+__device__ inline cdouble operator*(cdouble a, cdouble b) {
+  return {fma(a.x, b.x, -__dmul_rn(a.y, b.y)), fma(a.x, b.y, __dmul_rn(a.y, b.x))};
 }
 __host__ __device__ inline cfloat operator*(cfloat a, float s) { return {a.x * s, a.y * s}; }
 __host__ __device__ inline cdouble operator*(cdouble a, double s) { return {a.x * s, a.y * s}; }
@@ -251,7 +254,6 @@ __shared__ double g_exec_red[4][64];
 // own slot between passes.
 __shared__ int g_gemm_mode[4];
 
-//
 // TC: the executor of a kernel whose environment GEMMs may run on tcgen05 (the
 // BF16 form).  A kernel that holds tcgen05 instructions is given one block
 // per SM whatever its resources (the occupancy query's answer), so the other
@@ -262,10 +264,11 @@ struct CtaExecT {
   static constexpr bool tc = TC;
   __device__ int tid() const { return threadIdx.x; }
   __device__ int size() const { return blockDim.x; }
-  // threads among which the terms of a sum are dealt out: the same for every
-  // block size from 256, so that the results do not depend on it (the general
-  // QR and Jacobi of linalg.cuh deal to all threads; their plans have one size)
-  __device__ int sum_size() const { return min((int)blockDim.x, 256); }
+  // threads among which the terms of a sum are dealt out: those of a chain
+  // group, so that the results depend neither on the block size nor on the kernel
+  // form (the general QR and Jacobi of linalg.cuh deal to all threads; plans that
+  // reach them keep one form and size)
+  __device__ int sum_size() const { return 128; }
   __device__ int lane() const { return threadIdx.x & 31; }
   __device__ int warp() const { return threadIdx.x >> 5; }
   __device__ int nwarps() const { return blockDim.x >> 5; }

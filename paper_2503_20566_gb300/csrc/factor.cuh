@@ -558,7 +558,7 @@ __device__ __forceinline__ bool pair_rotation(typename Traits<T>::R& al, typenam
   const R gr = re(g), gi = im(g);
   R ga, iga;
   if constexpr (Traits<T>::cplx) {
-    const R g2 = gr * gr + gi * gi;
+    const R g2 = fmac(gr * gr, gi, gi);
     iga = jrsqrt1(g2);
     ga = g2 * iga;
     if (!(g2 > R(0))) return false;

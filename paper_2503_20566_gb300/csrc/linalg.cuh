@@ -132,11 +132,11 @@ __device__ inline void householder(T alpha, typename Traits<T>::R xn2, T& tau, T
     tau = zero<T>(); scal = zero<T>(); beta = alpha;
     return;
   }
-  R b = sqrt(ar * ar + ai * ai + xn2);
+  R b = sqrt(fmac(fmac(xn2, ai, ai), ar, ar));
   if (ar >= R(0)) b = -b;
   tau = make_scalar<T>((b - ar) / b, -ai / b);
   const R dr = ar - b, di = ai;
-  const R d2 = dr * dr + di * di;
+  const R d2 = fmac(dr * dr, di, di);
   scal = make_scalar<T>(dr / d2, -di / d2);
   beta = make_scalar<T>(b, R(0));
 }

@@ -63,7 +63,8 @@ def test_autotune_times_each_launch_once(per_sm, forms):
     assert per_sm > 2 or ctx.kernel_name != "gcf::vmc_kernel_grouped4"
 
 
-@pytest.mark.parametrize("prec,cplx,chi", [("fp64", True, 22), ("fp64", False, 43), ("fp32", False, 24)])
+@pytest.mark.parametrize("prec,cplx,chi", [("fp64", True, 22), ("fp64", False, 43), ("fp32", False, 24), ("fp32", True, 10),
+                                           ("fp32", True, 30), ("fp64", True, 10)])
 def test_amplitudes_do_not_depend_on_the_batch(prec, cplx, chi):
     """D_k = 3, bonds beyond the register factorisations in the first two (QR
     columns of 9 chi rows, Jacobi columns of 3 chi): the same bits alone, among
@@ -85,3 +86,50 @@ def test_amplitudes_do_not_depend_on_the_batch(prec, cplx, chi):
     ctx._check(ctx.lib.gcf_amplitude_noalloc(ctx.ctx, 3, _ptr(cfg), _ptr(la), _ptr(ph)), "noalloc")
     torch.cuda.synchronize()
     assert torch.equal(la, ref[0][:3]) and torch.equal(ph, ref[1][:3])
+
+
+def _two_lattices(prec, cplx, Dk, chi, sizes, n):
+    import paper_2503_20566_gb300 as G
+
+    ctxs, cfgs = [], []
+    for Lx, Ly in sizes:
+        lat, _, vals = oracle_net(Lx, Ly, 2, 2 * Dk, seed=81, complex_=cplx, precision=prec)
+        ctxs.append(G.Context(2, Lx, Ly, 2 * Dk, chi, g=0.4, complex_=cplx, precision=prec, seed=1))
+        ctxs[-1].set_tensors(vals)
+        cfgs.append(ctxs[-1].init_configs(n, None, synth.plaquette_powers(82, n, lat.n_plaquettes, 2)))
+    return ctxs, cfgs
+
+
+def _sampled(ctxs, cfgs, n):
+    import paper_2503_20566_gb300 as G
+
+    x = [c[:n].clone() for c in cfgs]
+    out = G.sample_multi(ctxs, x, 1, [7, 8])
+    return [t for a, o in zip(x, out) for t in (a, o["log_abs"], o["e_loc"].view(n, 2), o["O"].view(n, -1), o["accepted"])]
+
+
+def test_many_chains_of_several_lattices_share_ctas_and_keep_their_bits():
+    """Four chains per CTA from three rounds of one per CTA on (two CTAs fit an SM here)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ctxs, cfgs = _two_lattices("fp32", False, 2, 3, ((6, 5), (5, 6)), 3 * sms)
+    ref = None
+    for n, per_cta in ((3 * sms, 4), (3 * sms - 1, 1), (5, 1)):
+        got = _sampled(ctxs, cfgs, n)
+        assert ctxs[0].multi_chains_per_cta == per_cta, n
+        ref = ref or got
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b[:n]), n
+
+
+@pytest.mark.parametrize("prec,cplx,Dk,chi", [("fp32", False, 2, 24), ("tf32", False, 2, 24), ("bf16", False, 2, 16), ("fp32", True, 3, 10),
+                                              ("fp64", False, 2, 10), ("fp64", True, 2, 8)])
+def test_chains_are_the_same_one_or_four_per_cta(prec, cplx, Dk, chi, monkeypatch):
+    """Sums are dealt to 128 threads and products add in one order in every form."""
+    got = {}
+    for form, per_cta in (("cta", 1), ("group4", 4)):
+        monkeypatch.setenv("GCFVMC_MULTI", form)
+        ctxs, cfgs = _two_lattices(prec, cplx, Dk, chi, ((11, 6), (9, 7)) if chi > 12 else ((7, 6), (6, 5)), 9)
+        got[form] = _sampled(ctxs, cfgs, 9)
+        assert ctxs[0].multi_chains_per_cta == per_cta
+    for a, b in zip(got["cta"], got["group4"]):
+        assert torch.equal(a, b)
